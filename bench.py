@@ -514,9 +514,9 @@ def roofline(cls, prof, wl, sm_mhz, peaks, stats=None):
                "traffic": kernel_traffic("k_sweep<dfloat,8>", cells / max(1, n)),
                "traffic_per": f"launch of {cells / max(1, n):.0f} cell visits",
                "peak_source": f"hbm_gbs ({src})",
-               "note": "latency-bound: one visit is a chain of cluster reductions and Newton solves"}
+               "note": "latency-bound: one visit is two passes over the nodes around a chain of Newton solves"}
         if stats and stats.get("visits") and not is_cavity(wl):
-            out["latency_model"] = scan_latency_model(ms * 1e3 / cells, stats, peaks)
+            out["latency_model"] = scan_latency_model(ms * 1e3 / cells, stats, peaks, 1.0, 0.0)
         return out
     byts = 2 * K * 8 * wl.J * n
     ach = byts / (ms * 1e-3) / 1e9
@@ -524,14 +524,15 @@ def roofline(cls, prof, wl, sm_mhz, peaks, stats=None):
             "frac": ach / hbm["hbm_gbs"], "traffic": None, "peak_source": f"hbm_gbs ({src})"}
 
 
-def scan_latency_model(us_per_visit, stats, peaks):
-    """The scan's time per cell visit against the chain it runs: cluster reductions (two per
-    visit, then one per inner update) and Newton iterations (each an evaluation of the
-    separable Maxwellian with its combination and factorisation; one more evaluation per
-    solve that starts without one), at the latencies measured by sgs_probe_scan."""
+def scan_latency_model(us_per_visit, stats, peaks, per_visit=2.0, per_update=1.0):
+    """The scan's time per cell visit against the chain it runs: cluster reductions (per_visit
+    of them per visit and per_update per inner update; the scan kernels need one per visit and
+    none per update) and Newton iterations (each an evaluation of the separable Maxwellian with
+    its moments and direction; one more combination per solve), at the latencies measured by
+    sgs_probe_scan."""
     v = stats["visits"]
     inner = stats["inner_iters"] / v
-    reductions = 2.0 + inner
+    reductions = per_visit + per_update * inner
     evaluations = (stats["newton_iters"] + stats["newton_solves"]) / v
     t_red = reductions * peaks["scan_cluster_reduce_us"]
     t_newton = evaluations * peaks["scan_newton_iteration_us"]

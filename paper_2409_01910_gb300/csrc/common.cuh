@@ -30,6 +30,9 @@ struct InstDev {
   double b0;
   double bc_rho[4];      // inflow density (unused for diffuse walls)
   double wall_denom[4];  // sum over incoming v of w (v.n) Mhat_wall (diffuse walls)
+  double inv_dx, inv_dy, inv_eps;
+  double wall_scale[4];  // -w dv / wall_denom: diffuse-wall density per outgoing sum of (v.n / dv) f
+  double tol2_w;         // inner_tol^2 / w: the inner tolerance as an unweighted sum of squares
   double total_mass;
   double inner_tol;
   int inner_max, inner_fixed, inner_method, newton_max;
@@ -58,7 +61,7 @@ __host__ __device__ inline double node(int i, int N, double dv) { return (double
 // relative to the operands, enough for the cancellations of the cell equation, and run on the
 // FP32 pipes, which on this GPU have ~40x the FP64 throughput.
 // ---------------------------------------------------------------------------------------
-struct dfloat {
+struct __align__(8) dfloat {
   float hi, lo;
 };
 
@@ -89,16 +92,15 @@ __device__ __forceinline__ dfloat& operator-=(dfloat& a, dfloat b) { return a = 
 // hi keeps the leading 24 significand bits (truncated), lo the next bits rounded to 24.
 // Magnitudes below 2^-100 (irrelevant next to the O(1) values they are summed with) map to 0.
 __device__ __forceinline__ dfloat df_split(double x) {
-  unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  unsigned int sign = (unsigned int)(u >> 63) << 31;
-  int e = (int)((u >> 52) & 0x7ff) - 1023;
+  const unsigned int h = (unsigned int)__double2hiint(x), l = (unsigned int)__double2loint(x);
+  const int e = (int)((h >> 20) & 0x7ffu) - 1023;
   if (e < -100) return {0.0f, 0.0f};
-  unsigned long long m = (u & 0xfffffffffffffULL) | 0x10000000000000ULL;  // 53-bit significand
-  unsigned int mh = (unsigned int)(m >> 29);                               // top 24 bits
-  float hi = __int_as_float((int)(sign | ((unsigned int)(e + 127) << 23) | (mh & 0x7fffff)));
-  unsigned int ml = (unsigned int)(m & 0x1fffffffULL);                     // low 29 bits
-  float lo = ldexpf((float)ml, e - 52);
-  return {hi, sign ? -lo : lo};
+  const unsigned int sign = h & 0x80000000u;
+  const float hi = __uint_as_float(sign | ((unsigned int)(e + 127) << 23) | ((h & 0xfffffu) << 3) | (l >> 29));
+  // low 29 bits as a fraction of the last place of hi, 2^(e - 23), which is a normal number
+  const float ulp = __uint_as_float(sign | ((unsigned int)(e + 104) << 23));
+  const float lo = __uint2float_rn(l & 0x1fffffffu) * 1.862645149230957e-09f * ulp;
+  return {hi, lo};
 }
 
 // exp in double-float arithmetic (no FP64 instruction): Cody and Waite's additive argument

@@ -221,17 +221,18 @@ struct SweepShape {
 // arithmetic of the sweep's elementwise work and reductions
 constexpr int kSweepF64 = 0;   // native FP64
 constexpr int kSweepDF64 = 1;  // double-float on the FP32 pipes (FP64-class accuracy)
-constexpr int kSweepF32 = 2;   // plain FP32 (converges only to FP32 resolution)
 SweepShape sweep_shape(int N, int arith);
 bool sweep_shape_valid(int N, const SweepShape& sh);
 // Sweep launch shapes: nodes per thread with a compiled kernel, and the number of clusters of
 // the shape that fit on the device at once (0: the shape cannot run).
 bool sweep_ept_compiled(int ept);
-cudaError_t sweep_max_clusters(const SweepShape& sh, int arith, int* n);
+cudaError_t sweep_max_clusters(int N, const SweepShape& sh, int arith, int* n);
 // 2-D: one wavefront (anti-diagonal wf of ordering 0..3) of the single 2-D instance.
 cudaError_t launch_sweep2d(const SweepArgs& a, const SweepShape& sh, int arith, int ordering, int wf, int ncells,
                            cudaStream_t st);
 cudaError_t launch_sweep(const SweepArgs& a, const SweepShape& sh, int arith, cudaStream_t st);
+// The double-float scan of sgs_dc_step (sweep_nodes.cu).
+cudaError_t launch_sweep_nodes(const SweepArgs& a, const SweepShape& sh, cudaStream_t st);
 // Fast (Carleman-form) spectral operator on the tensor cores (fast.cu): one chunk of S slots
 // (half-sphere nodes, the loss slot last) for every cell.
 struct FastArgs {

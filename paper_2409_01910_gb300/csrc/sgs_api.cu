@@ -113,6 +113,7 @@ struct sgs_handle {
   } off;
   int cproj = 0;  // conservation projection of Q after every spectral collision step (mode 1 or 2)
   bool order2 = false;  // second-order reconstruction (1-D)
+  bool dc_scan = false;  // within sgs_dc_step's iterations (1-D): scans keep the node-wise kernel
   bool dc_ref = false;  // FP32 collisions use the increment form against the stored reference
   int dc_prec = SGS_DF64;  // arithmetic of the high-precision evaluation in sgs_dc_step
   bool two_d = false;      // 2-D space: one instance, wavefront scans, four orderings
@@ -445,6 +446,10 @@ void sgs::fill_inst(const sgs_problem& p, int N, double dv, InstDev& I) {
   I.newton_max = p.newton_max;
   I.newton_tol = p.newton_tol;
   double w = dv * dv * dv;
+  I.inv_dx = 1.0 / I.dx;
+  I.inv_dy = 1.0 / I.dy;
+  I.inv_eps = 1.0 / p.eps;
+  I.tol2_w = p.inner_tol * p.inner_tol / w;
   for (int s = 0; s < (two_d ? 4 : 2); s++) {
     const sgs_bc& b = p.bc[s];
     const int dn = s < 2 ? 0 : 1;  // normal velocity component of the side
@@ -468,6 +473,7 @@ void sgs::fill_inst(const sgs_problem& p, int N, double dv, InstDev& I) {
     for (int d = 0; d < 3; d++)
       for (int i = 0; i < N; i++) sd[d] += (d == dn ? node(i, N, dv) : 1.0) * I.wall[s][d][i];
     I.wall_denom[s] = w * sd[0] * sd[1] * sd[2];
+    I.wall_scale[s] = -w * dv / I.wall_denom[s];
   }
 }
 
@@ -794,7 +800,8 @@ int sweep_impl(sgs_handle* h, double* f, const double* P, const double* rhs, int
     if (e != cudaSuccess) return cuda_status(e);
     a.rhs = b2;
   }
-  return cuda_status(launch_sweep(a, h->sweep, h->sweep_arith, st));
+  return cuda_status(h->dc_scan ? launch_sweep_nodes(a, h->sweep, st)
+                                : launch_sweep(a, h->sweep, h->sweep_arith, st));
 }
 
 int rescale_impl(sgs_handle* h, double* f, cudaStream_t st) {
@@ -1377,11 +1384,13 @@ int sgs_dc_step(sgs_handle* h, double* f, double* Q, double* P, int lo_iters, do
   // P is the next iteration's), so every collision step overlaps a scan; otherwise the next
   // iteration evaluates it first.
   const bool ov = overlap_ok(h, 0);
-  for (int it = 0; it < lo_iters; it++) {
+  h->dc_scan = !h->two_d;
+  for (int it = 0; it < lo_iters && r == SGS_OK; it++) {
     int fl = ov ? SGS_IT_P_VALID | SGS_IT_EVAL : (it == 0 ? SGS_IT_P_VALID : 0);
-    if ((r = iterate_impl(h, f, Q, P, nullptr, fl, nullptr, st))) return r;
+    r = iterate_impl(h, f, Q, P, nullptr, fl, nullptr, st);
   }
-  return SGS_OK;
+  h->dc_scan = false;
+  return r;
 }
 
 int sgs_set_dc_precision(sgs_handle* h, int precision) {
@@ -1447,7 +1456,7 @@ int sgs_set_sweep_shape(sgs_handle* h, int ept, int cluster, int threads) {
   SweepShape sh{ept, cluster, threads};
   if (!sweep_ept_compiled(ept) || !sweep_shape_valid(h->N, sh)) return SGS_ERR_ARG;
   int n = 0;
-  cudaError_t e = sweep_max_clusters(sh, h->sweep_arith, &n);
+  cudaError_t e = sweep_max_clusters(h->N, sh, h->sweep_arith, &n);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return SGS_ERR_UNSUPPORTED;
@@ -1479,7 +1488,7 @@ int sgs_autotune(sgs_handle* h, double* f, const double* P, int reps, sgs_tuning
       if (!sweep_shape_valid(h->N, sh)) continue;
       if ((long long)(tpb - 32) * cs * ept >= K && tpb > 160) continue;  // a whole warp idle in every CTA
       int n = 0;
-      if (sweep_max_clusters(sh, h->sweep_arith, &n) != cudaSuccess) {
+      if (sweep_max_clusters(h->N, sh, h->sweep_arith, &n) != cudaSuccess) {
         cudaGetLastError();
         continue;
       }
