@@ -245,6 +245,7 @@ __global__ void __launch_bounds__(256) k_dft_i1(SpecBufs<T> sb, int N) {
   __syncthreads();
   T scale = (T)(1.0 / ((double)N * N * N));
   int g = c / kLanes, lane = c % kLanes;
+  const int ls = g == sb.fold_group ? sb.fold_lanes : kLanes;  // lanes of the group's rows (SpecBufs)
   for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
     int k1 = t / n, k3 = t % n;
     T ar = 0, ai = 0, br = 0, bi = 0;
@@ -256,60 +257,133 @@ __global__ void __launch_bounds__(256) k_dft_i1(SpecBufs<T> sb, int N) {
       br += b.x * co - b.y * si;
       bi += b.x * si + b.y * co;
     }
-    long long o = ((((long long)g * n + k1) * n + k2) * n + k3) * kLanes + lane;
+    long long o = (long long)g * n * n * n * kLanes + (((long long)k1 * n + k2) * n + k3) * ls + lane;
     sb.ahat[o] = make_cplx(ar * scale, ai * scale);
     sb.bhat[o] = make_cplx(br * scale, bi * scale);
   }
 }
 
 // ---------------------------------------------------------------------------------------
-// Direct spectral sum. Work unit = one output row (k1, k2) of the Hermitian half and a
-// range of m1; a step = one (m1, m2) with its weight block W[(m3, k3) valid pairs]
-// precomputed at setup in exactly the loop order below. Each warp owns one group of 32
-// cells (lane = cell) and accumulates the 2H+1 outputs k3 of the row in registers; the
-// rows ahat[(k1-m1, k2-m2, .)] and bhat[(m1, m2, .)] and the weight block of the next
-// step are brought in by bulk copies into shared memory while the current step computes.
-// FP32 keeps both rows in registers (full unroll, weights read as warp-uniform shared
-// loads); FP64 reads them from shared memory.
+// Direct spectral sum. Work unit = one output row (k1, k2) of the Hermitian half and a range of
+// m1; a step = one (m1, m2) with its weights, the rows ahat[(k1-m1, k2-m2, .)] and
+// bhat[(m1, m2, .)], brought into shared memory by bulk copies while the previous step
+// computes. Lane = cell (a lane group of 32 cells per four warps).
+//
+// With N = 4 BK the n = 4 BK - 1 outputs k3 and inputs m3 of a step fall into four blocks of BK
+// (the last one short by one). Warp kb of a lane group accumulates the outputs of block kb in
+// registers and walks the blocks c of m3: |kb - c| <= 1 is a full BK x BK square of valid pairs
+// (|k3 - m3| <= H), |kb - c| = 2 a triangle, |kb - c| = 3 empty. Along m3 the BK values of ahat
+// that meet the outputs slide by one, so a thread loads one value of each row per m3 and keeps
+// the window in registers (its slots rotate; the loop is unrolled by BK). This replaces a
+// fully unrolled step of 721 pairs per warp with both rows in registers (FP32), which was bound
+// by instruction fetch (69 KB of code) at 255 registers and two warps per scheduler, and a
+// version with two shared loads per pair (FP64), whose 127 KB of rows for two warps left half
+// of an SM's schedulers idle. Measured: FP32,
+// 32 cells of 32^3, 1.62 -> 1.55 ms (42 TFLOP/s; 64 registers, 20 warps per SM; now held by
+// operand dispatch, 0.7 stalls per issue); FP64 is at 0.87 of the DFMA rate times 10 flops in 6
+// instructions, its cap. FP32 in packed pairs (fma.rn.f32x2 on outputs i, i + 1) took 1.94 ms: about
+// one move per packed operand.
+// Four warps do 3/14, 4/14, 4/14, 3/14 of the blocks; every other lane group (or block) takes
+// them in the order 1, 0, 3, 2, so that the SM's schedulers get the same work.
+// Each output is summed over m1, m2, m3 in ascending order in the arithmetic T, as before.
 // ---------------------------------------------------------------------------------------
-template <typename T, int H>
-__global__ void __launch_bounds__(128) k_sum(SumArgs<T> a) {
+constexpr int kSumBlocksPerStep = 14;  // blocks of (k3, m3) pairs of a step
+
+// Weights of a step: the valid blocks (kb, c), kb major, c ascending, each [m3][k3] of BK x BK
+// (zero where the pair is not valid).
+__host__ __device__ constexpr int sum_first_block(int kb) { return kb == 0 ? 0 : (kb == 1 ? 3 : (kb == 2 ? 7 : 11)); }
+__host__ __device__ constexpr int sum_weights(int BK) { return kSumBlocksPerStep * BK * BK; }
+
+// Weight row of one m3: BK consecutive values by the widest aligned loads.
+template <typename T, int BK>
+__device__ __forceinline__ void load_weights(const T* p, T (&w)[BK]) {
+  constexpr int V = (BK % 4 == 0 && sizeof(T) == 4) ? 4 : (BK % 2 == 0 ? 2 : 1);
+#pragma unroll
+  for (int i = 0; i < BK; i += V) {
+    if constexpr (V == 4) {
+      const float4 x = *reinterpret_cast<const float4*>(p + i);
+      w[i] = x.x, w[i + 1] = x.y, w[i + 2] = x.z, w[i + 3] = x.w;
+    } else if constexpr (V == 2) {
+      const typename CplxOf<T>::type x = *reinterpret_cast<const typename CplxOf<T>::type*>(p + i);
+      w[i] = x.x, w[i + 1] = x.y;
+    } else {
+      w[i] = p[i];
+    }
+  }
+}
+
+// One block of a step for one warp. KIND 0: full; -1: the block below the band (kb - c = 2, pairs
+// i < u); +1: above it (kb - c = -2, pairs i > u). win: the sliding window of ahat, slot
+// (i - u) mod BK; ra: ahat of (k3 = first output, m3 = first input of the block), rb: bhat of
+// that m3 (both already at this lane).
+template <int KIND, typename T, int BK, int LS>
+__device__ __forceinline__ void sum_block(const T* w, const typename CplxOf<T>::type* ra,
+                                          const typename CplxOf<T>::type* rb, bool k_pad, bool m_pad,
+                                          typename CplxOf<T>::type (&win)[BK], T (&accr)[BK], T (&acci)[BK]) {
   typedef typename CplxOf<T>::type CT;
-  constexpr int n = 2 * H + 1;
-  constexpr int NP = 3 * H * H + 3 * H + 1;
+  // FP64 skips the pairs of the padding output and input (k_pad, m_pad: this block has them); for
+  // FP32 their zero weights cost less than the test
+  constexpr bool kSkip = sizeof(T) == 8;
+#pragma unroll
+  for (int u = 0; u < BK; u++) {
+    if (KIND == 0 || (KIND < 0 && u > 0)) win[(BK - u) % BK] = ra[-u * LS];
+    if (kSkip && u == BK - 1 && m_pad) break;
+    const CT bv = rb[u * LS];
+    T wv[BK];
+    load_weights<T, BK>(w + u * BK, wv);
+#pragma unroll
+    for (int i = 0; i < BK; i++) {
+      if ((KIND < 0 && i >= u) || (KIND > 0 && i <= u)) continue;
+      if (kSkip && i == BK - 1 && k_pad) break;
+      const CT av = win[(i - u + BK) % BK];
+      const T br = wv[i] * bv.x, bi = wv[i] * bv.y;
+      accr[i] = fma(av.x, br, accr[i]);
+      accr[i] = fma(-av.y, bi, accr[i]);
+      acci[i] = fma(av.x, bi, acci[i]);
+      acci[i] = fma(av.y, br, acci[i]);
+    }
+  }
+}
+
+// F > 1 (FP64, a last lane group of at most 32 / F cells): the group's rows hold 32 / F lanes, and
+// the F parts of a warp take F consecutive steps at a time, summed at the end. The FP64 pipe
+// works through all 32 lanes whether they hold a cell or not: 40 cells of 24^3 took as long as
+// 64 (collision step 22.1 ms, folded 15.0).
+template <typename T, int BK, int F>
+__global__ void __launch_bounds__(512) k_sum(SumArgs<T> a) {
+  typedef typename CplxOf<T>::type CT;
+  constexpr int H = 2 * BK - 1, n = 4 * BK - 1;
   constexpr int VEC = 16 / (int)sizeof(T);
-  constexpr int PW = (NP + VEC - 1) / VEC * VEC;
-  constexpr bool kRegs = sizeof(T) == 4;
-  constexpr int kRowBufs = kRegs ? 1 : 2;
-  typedef typename VecOf<T>::type VT;
+  constexpr int PW = (sum_weights(BK) + VEC - 1) / VEC * VEC;
+  constexpr int PWS = PW + (F > 1 ? VEC : 0);      // the parts' weights start in different banks
+  constexpr int LS = kLanes / F;                   // lanes of a row
+  constexpr int kRow = n * LS;                     // ahat row; the bhat row has one more, of zeros
+  constexpr int kRows = kRow + (n + 1) * LS;
   extern __shared__ __align__(128) unsigned char smraw[];
-  T* Wb = (T*)smraw;                                   // [2][PW]
-  CT* rows = (CT*)(smraw + 2 * PW * sizeof(T));        // [kRowBufs][NW][2][n][32]
+  T* Wb = (T*)smraw;                                   // [2][F][PWS]
+  CT* rows = (CT*)(smraw + 2 * F * PWS * sizeof(T));   // [2][NG][F][kRows]
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ int s_err;
 
-  const int NW = blockDim.x >> 5;
+  const int NG = blockDim.x >> 7;       // lane groups of a block, four warps each
   const int4 ud = a.units[blockIdx.x];  // k1, k2, m1_lo, m1_hi
   const long long step0 = a.unit_step0[blockIdx.x];
   const int k1 = ud.x, k2 = ud.y, m1lo = ud.z, m1hi = ud.w;
   const int m2lo = max(-H, k2 - H), m2hi = min(H, k2 + H);
   const int nm2 = m2hi - m2lo + 1;
   const int S = (m1hi - m1lo + 1) * nm2;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g0 = blockIdx.y * NW;
-  const int ng = min(NW, a.G - g0);
-  const uint32_t row_bytes = n * kLanes * sizeof(CT);
-  const uint32_t stage_bytes = PW * sizeof(T) + ng * 2 * row_bytes;
+  const int B = (S + F - 1) / F;        // batches of F steps
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = warp >> 2;
+  const int part = lane / LS, cell = lane % LS;
+  const int kb = ((grp + blockIdx.x) & 1) ? ((warp & 3) ^ 1) : (warp & 3);
+  const int g0 = a.g0 + blockIdx.y * NG;
+  const int ng = min(NG, a.G - g0);
+  const uint32_t row_bytes = kRow * sizeof(CT);
 
   if (a.active) {
     // a block whose lane groups hold no cell of an active instance has nothing to compute
-    __shared__ int s_any;
-    if (threadIdx.x == 0) s_any = 0;
-    __syncthreads();
-    const int c = (g0 + warp) * kLanes + lane;
-    if (warp < ng && c < a.C && a.active[a.cell_inst[c]]) s_any = 1;
-    __syncthreads();
-    if (!s_any) return;
+    const int c = (g0 + grp) * kLanes + cell;
+    if (!__syncthreads_or(grp < ng && c < a.C && a.active[a.cell_inst[c]])) return;
   }
   if (threadIdx.x == 0) {
     mbar_init(&bar[0], 1);
@@ -317,97 +391,68 @@ __global__ void __launch_bounds__(128) k_sum(SumArgs<T> a) {
     s_err = 0;
     fence_mbar_init();
   }
+  for (int t = threadIdx.x; t < 2 * NG * F * LS; t += blockDim.x)
+    rows[(t / LS + 1) * kRows - LS + t % LS] = make_cplx((T)0, (T)0);
   __syncthreads();
 
-  auto issue = [&](int s) {
-    int m1 = m1lo + s / nm2, m2 = m2lo + s % nm2;
-    int b = s & 1;
-    mbar_arrive_expect_tx(&bar[b], stage_bytes);
-    bulk_g2s(Wb + b * PW, a.W + (step0 + s) * PW, PW * sizeof(T), &bar[b]);
-    int rb = kRegs ? 0 : b;
-    for (int w = 0; w < ng; w++) {
-      long long ga = (((long long)(g0 + w) * n + (k1 - m1 + H)) * n + (k2 - m2 + H)) * n * kLanes;
-      long long gb = (((long long)(g0 + w) * n + (m1 + H)) * n + (m2 + H)) * n * kLanes;
-      CT* dst = rows + ((rb * NW + w) * 2) * n * kLanes;
-      bulk_g2s(dst, a.ahat + ga, row_bytes, &bar[b]);
-      bulk_g2s(dst + n * kLanes, a.bhat + gb, row_bytes, &bar[b]);
+  auto issue = [&](int bt) {
+    const int b = bt & 1, nf = min(F, S - bt * F);
+    mbar_arrive_expect_tx(&bar[b], nf * (PW * sizeof(T) + ng * 2 * row_bytes));
+    for (int h = 0; h < nf; h++) {
+      const int s = bt * F + h, m1 = m1lo + s / nm2, m2 = m2lo + s % nm2;
+      bulk_g2s(Wb + (b * F + h) * PWS, a.W + (step0 + s) * PW, PW * sizeof(T), &bar[b]);
+      for (int w = 0; w < ng; w++) {
+        const long long ga = (((long long)(k1 - m1 + H)) * n + (k2 - m2 + H)) * kRow;
+        const long long gb = (((long long)(m1 + H)) * n + (m2 + H)) * kRow;
+        const long long g = (long long)(g0 + w) * n * n * n * kLanes;
+        CT* dst = rows + ((b * NG + w) * F + h) * kRows;
+        bulk_g2s(dst, a.ahat + g + ga, row_bytes, &bar[b]);
+        bulk_g2s(dst + kRow, a.bhat + g + gb, row_bytes, &bar[b]);
+      }
     }
   };
 
-  if (threadIdx.x == 0 && S > 0) issue(0);
+  if (threadIdx.x == 0 && B > 0) issue(0);
 
-  T accr[n], acci[n];
+  T accr[BK], acci[BK];
 #pragma unroll
-  for (int i = 0; i < n; i++) accr[i] = acci[i] = (T)0;
+  for (int i = 0; i < BK; i++) accr[i] = acci[i] = (T)0;
 
-  const bool active = warp < ng;
+  const bool active = grp < ng;
   int fail_b = 0, fail_par = 0;
-  for (int s = 0; s < S; s++) {
+  for (int s = 0; s < B; s++) {
     const int b = s & 1;
     if (!mbar_wait(&bar[b], (s >> 1) & 1, a.spin_max)) {
       s_err = 1;
       fail_b = b;
       fail_par = (s >> 1) & 1;
     }
-    const VT* W4 = (const VT*)(Wb + b * PW);
-    if (kRegs) {
-      CT Ar[n], Br[n];
-      const CT* rw = rows + (warp * 2) * n * kLanes;
-      if (active) {
+    __syncthreads();
+    if (s_err) break;
+    // the other buffer was released by the barrier above: the next batch goes into it
+    if (threadIdx.x == 0 && s + 1 < B) issue(s + 1);
+    if (active && s * F + part < S) {
+      // ahat of l = k3 - m3 is at l + H = BK (kb - c) + 2 BK - 1 + i - u
+      const CT* ra = rows + ((b * NG + grp) * F + part) * kRows + (kb * BK + 2 * BK - 1) * LS + cell;
+      const CT* rb = rows + ((b * NG + grp) * F + part) * kRows + kRow + cell;
+      const T* w = Wb + (b * F + part) * PWS + sum_first_block(kb) * BK * BK;
+      CT win[BK];
+      int c = max(0, kb - 1);
+      if (kb >= 2) {
+        const int cl = kb - 2;
+        sum_block<-1, T, BK, LS>(w, ra - cl * BK * LS, rb + cl * BK * LS, kb == 3, false, win, accr, acci);
+        w += BK * BK;
+      } else {
 #pragma unroll
-        for (int i = 0; i < n; i++) {
-          Ar[i] = rw[i * kLanes + lane];
-          Br[i] = rw[(n + i) * kLanes + lane];
-        }
+        for (int i = 1; i < BK; i++) win[i] = ra[i * LS];
       }
-      __syncthreads();
-      if (s_err) break;
-      if (threadIdx.x == 0 && s + 1 < S) issue(s + 1);
-      if (active) {
-        VT wv;
-        int p = 0;
-#pragma unroll
-        for (int m3 = -H; m3 <= H; m3++) {
-          const CT bv = Br[m3 + H];
-#pragma unroll
-          for (int k3 = (m3 - H > -H ? m3 - H : -H); k3 <= (m3 + H < H ? m3 + H : H); k3++) {
-            if (p % VEC == 0) wv = W4[p / VEC];
-            const T w = vec_get(wv, p % VEC);
-            p++;
-            const CT av = Ar[k3 - m3 + H];
-            const T br = w * bv.x, bi = w * bv.y;
-            accr[k3 + H] = fma(av.x, br, accr[k3 + H]);
-            accr[k3 + H] = fma(-av.y, bi, accr[k3 + H]);
-            acci[k3 + H] = fma(av.x, bi, acci[k3 + H]);
-            acci[k3 + H] = fma(av.y, br, acci[k3 + H]);
-          }
-        }
+      const int c1 = min(3, kb + 1);
+#pragma unroll 1
+      for (; c <= c1; c++) {
+        sum_block<0, T, BK, LS>(w, ra - c * BK * LS, rb + c * BK * LS, kb == 3, c == 3, win, accr, acci);
+        w += BK * BK;
       }
-    } else {
-      __syncthreads();
-      if (s_err) break;
-      if (threadIdx.x == 0 && s + 1 < S) issue(s + 1);
-      if (active) {
-        const CT* rw = rows + ((b * NW + warp) * 2) * n * kLanes;
-        VT wv;
-        int p = 0;
-#pragma unroll
-        for (int m3 = -H; m3 <= H; m3++) {
-          const CT bv = rw[(n + m3 + H) * kLanes + lane];
-#pragma unroll
-          for (int k3 = (m3 - H > -H ? m3 - H : -H); k3 <= (m3 + H < H ? m3 + H : H); k3++) {
-            if (p % VEC == 0) wv = W4[p / VEC];
-            const T w = vec_get(wv, p % VEC);
-            p++;
-            const CT av = rw[(k3 - m3 + H) * kLanes + lane];
-            const T br = w * bv.x, bi = w * bv.y;
-            accr[k3 + H] = fma(av.x, br, accr[k3 + H]);
-            accr[k3 + H] = fma(-av.y, bi, accr[k3 + H]);
-            acci[k3 + H] = fma(av.x, bi, acci[k3 + H]);
-            acci[k3 + H] = fma(av.y, br, acci[k3 + H]);
-          }
-        }
-      }
+      if (kb < 2) sum_block<1, T, BK, LS>(w, ra, rb + c * BK * LS, false, c == 3, win, accr, acci);
     }
   }
   if (s_err) {
@@ -419,24 +464,33 @@ __global__ void __launch_bounds__(128) k_sum(SumArgs<T> a) {
     }
     return;
   }
-  if (active) {
-    CT* out = a.partial + ((long long)blockIdx.x * a.Gs + (g0 + warp)) * n * kLanes;
+  if (F > 1) {
 #pragma unroll
-    for (int i = 0; i < n; i++) out[i * kLanes + lane] = make_cplx(accr[i], acci[i]);
+    for (int i = 0; i < BK; i++)
+#pragma unroll
+      for (int o = LS; o < kLanes; o <<= 1) {
+        accr[i] += __shfl_xor_sync(0xffffffffu, accr[i], o);
+        acci[i] += __shfl_xor_sync(0xffffffffu, acci[i], o);
+      }
+  }
+  if (active) {
+    CT* out = a.partial + ((long long)blockIdx.x * a.Gs + (g0 + grp)) * n * kLanes;
+#pragma unroll
+    for (int i = 0; i < BK; i++)
+      if (kb * BK + i < n) out[(kb * BK + i) * kLanes + lane] = make_cplx(accr[i], acci[i]);
   }
 }
 
 // ---------------------------------------------------------------------------------------
 // Direct spectral sum in double-float arithmetic on the FP32 pipes (the high-precision
-// evaluation of the defect correction). Same units, steps and weight order as k_sum; the
+// evaluation of the defect correction). Same units, steps, blocks and weight order as k_sum; the
 // transformed rows arrive split into (hi, lo) float pairs (k_split_spec) and the weights as
 // the FP32 table (hi) plus its FP32 remainder table (lo). Products are formed exactly in
 // their leading part (FMA two-product) with first-order cross terms, and accumulated by
 // error-free two-sums into (hi, lo) accumulators, so each term carries about 2^-48 relative
-// error instead of FP32's 2^-24.
-// One block of KW warps serves one group of 32 cells (lane = cell); warp w accumulates the
-// outputs k3 = -H + w + KW j. Rows and weights are double-buffered in shared memory by
-// bulk copies, as in k_sum.
+// error instead of FP32's 2^-24. Bound by the FP32 pipes (56 operations per pair): 32 cells of
+// 32^3 in 11.3 ms, 0.77 of the pipes' rate (13.1 ms with outputs strided over the warps, two
+// shared loads and a range test per pair).
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ void df_mul_acc(float xh, float xl, float yh, float yl, float& ah, float& al) {
   // (ah, al) += (xh + xl)(yh + yl), to first order in the low parts
@@ -451,15 +505,54 @@ __device__ __forceinline__ void df_mul_acc(float xh, float xl, float yh, float y
   al += err + e;
 }
 
-template <int H, int KW>
-__global__ void __launch_bounds__(KW * 32, 2) k_sum_df(SumDfArgs a) {
-  constexpr int n = 2 * H + 1;
-  constexpr int NP = 3 * H * H + 3 * H + 1;
-  constexpr int PW = (NP + 3) / 4 * 4;
-  constexpr int NJ = (n + KW - 1) / KW;  // outputs per warp
+// Side of a square of the double-float sum: half a block where it divides (8 warps per lane
+// group), which keeps the unrolled body (56 operations a pair) within the instruction cache:
+// with whole blocks of N = 32 it is 121 KB of code and twice as slow.
+__host__ __device__ constexpr int df_side(int BK) { return BK % 2 == 0 ? BK / 2 : BK; }
+
+// One HB x HB square (KIND as in sum_block); rows of the weights are BK apart.
+template <int KIND, int BK, int HB>
+__device__ __forceinline__ void sum_block_df(const float* wh, const float* wl, const float4* ra, const float4* rb,
+                                             float4 (&win)[HB], float (&rh)[HB], float (&rl)[HB], float (&ih)[HB],
+                                             float (&il)[HB]) {
+#pragma unroll
+  for (int u = 0; u < HB; u++) {
+    if (KIND == 0 || (KIND < 0 && u > 0)) win[(HB - u) % HB] = ra[-u * kLanes];
+    const float4 bv = rb[u * kLanes];
+    float h[HB], l[HB];
+    load_weights<float, HB>(wh + u * BK, h);
+    load_weights<float, HB>(wl + u * BK, l);
+#pragma unroll
+    for (int i = 0; i < HB; i++) {
+      if ((KIND < 0 && i >= u) || (KIND > 0 && i <= u)) continue;
+      const float4 av = win[(i - u + HB) % HB];
+      // w b = (w b_re, w b_im), leading parts exact
+      float brh = h[i] * bv.x, brl = fmaf(h[i], bv.x, -brh);
+      brl = fmaf(h[i], bv.y, brl);
+      brl = fmaf(l[i], bv.x, brl);
+      float bih = h[i] * bv.z, bil = fmaf(h[i], bv.z, -bih);
+      bil = fmaf(h[i], bv.w, bil);
+      bil = fmaf(l[i], bv.z, bil);
+      // a (w b): re += a_re br - a_im bi, im += a_re bi + a_im br
+      df_mul_acc(av.x, av.y, brh, brl, rh[i], rl[i]);
+      df_mul_acc(-av.z, -av.w, bih, bil, rh[i], rl[i]);
+      df_mul_acc(av.x, av.y, bih, bil, ih[i], il[i]);
+      df_mul_acc(av.z, av.w, brh, brl, ih[i], il[i]);
+    }
+  }
+}
+
+template <int BK>
+__global__ void __launch_bounds__(128 * (BK / df_side(BK)), 2) k_sum_df(SumDfArgs a) {
+  constexpr int H = 2 * BK - 1, n = 4 * BK - 1;
+  constexpr int HB = df_side(BK), per = BK / HB;  // squares of HB; per block side
+  constexpr int NB = 4 * per, D = 2 * per;         // squares along a row; |kb - c| = D is the triangle
+  constexpr int PW = (sum_weights(BK) + 3) / 4 * 4;
+  constexpr int kRow = n * kLanes;
+  constexpr int kRows = kRow + (n + 1) * kLanes;
   extern __shared__ __align__(128) unsigned char smraw[];
-  float* Wb = (float*)smraw;                            // [2][2][PW]: buffer, (hi, lo)
-  float4* rows = (float4*)(smraw + 4 * PW * sizeof(float));  // [2][2][n][32]: buffer, (a, b)
+  float* Wb = (float*)smraw;                                 // [2][2][PW]: buffer, (hi, lo)
+  float4* rows = (float4*)(smraw + 4 * PW * sizeof(float));  // [2][kRows]: buffer, (a, b)
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ int s_err;
 
@@ -470,8 +563,10 @@ __global__ void __launch_bounds__(KW * 32, 2) k_sum_df(SumDfArgs a) {
   const int nm2 = m2hi - m2lo + 1;
   const int S = (m1hi - m1lo + 1) * nm2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // warps kb and kb + 4 share a scheduler and have 11 full squares between them for every kb
+  const int kb = warp;
   const int g = blockIdx.y;
-  const uint32_t row_bytes = n * kLanes * sizeof(float4);
+  const uint32_t row_bytes = kRow * sizeof(float4);
   const uint32_t stage_bytes = 2 * PW * sizeof(float) + 2 * row_bytes;
 
   if (a.active) {
@@ -487,6 +582,7 @@ __global__ void __launch_bounds__(KW * 32, 2) k_sum_df(SumDfArgs a) {
     s_err = 0;
     fence_mbar_init();
   }
+  if (warp < 2) rows[warp * kRows + kRows - kLanes + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   __syncthreads();
 
   auto issue = [&](int s) {
@@ -495,18 +591,18 @@ __global__ void __launch_bounds__(KW * 32, 2) k_sum_df(SumDfArgs a) {
     mbar_arrive_expect_tx(&bar[b], stage_bytes);
     bulk_g2s(Wb + (2 * b) * PW, a.Whi + (step0 + s) * PW, PW * sizeof(float), &bar[b]);
     bulk_g2s(Wb + (2 * b + 1) * PW, a.Wlo + (step0 + s) * PW, PW * sizeof(float), &bar[b]);
-    long long ga = (((long long)g * n + (k1 - m1 + H)) * n + (k2 - m2 + H)) * n * kLanes;
-    long long gb = (((long long)g * n + (m1 + H)) * n + (m2 + H)) * n * kLanes;
-    float4* dst = rows + (2 * b) * n * kLanes;
+    long long ga = (((long long)g * n + (k1 - m1 + H)) * n + (k2 - m2 + H)) * kRow;
+    long long gb = (((long long)g * n + (m1 + H)) * n + (m2 + H)) * kRow;
+    float4* dst = rows + b * kRows;
     bulk_g2s(dst, a.ahat + ga, row_bytes, &bar[b]);
-    bulk_g2s(dst + n * kLanes, a.bhat + gb, row_bytes, &bar[b]);
+    bulk_g2s(dst + kRow, a.bhat + gb, row_bytes, &bar[b]);
   };
 
   if (threadIdx.x == 0 && S > 0) issue(0);
 
-  float rh[NJ], rl[NJ], ih[NJ], il[NJ];
+  float rh[HB], rl[HB], ih[HB], il[HB];
 #pragma unroll
-  for (int j = 0; j < NJ; j++) rh[j] = rl[j] = ih[j] = il[j] = 0.0f;
+  for (int j = 0; j < HB; j++) rh[j] = rl[j] = ih[j] = il[j] = 0.0f;
 
   int fail_b = 0, fail_par = 0;
   for (int s = 0; s < S; s++) {
@@ -520,39 +616,31 @@ __global__ void __launch_bounds__(KW * 32, 2) k_sum_df(SumDfArgs a) {
     if (s_err) break;
     // the other buffer was released by the barrier above: prefetch the next step into it
     if (threadIdx.x == 0 && s + 1 < S) issue(s + 1);
-    const float* Wh = Wb + (2 * b) * PW;
-    const float* Wl = Wh + PW;
-    const float4* ra = rows + (2 * b) * n * kLanes;
-    const float4* rb = ra + n * kLanes;
-    int off = 0;  // first weight of the current m3 in the packed (m3, k3) order
-    // m3 stays a loop (the body, unrolled over the warp's outputs, is long enough to
-    // hide latency; unrolling m3 as well overflows the instruction cache)
-#pragma unroll 1
-    for (int m3 = -H; m3 <= H; m3++) {
-      const int lo = m3 - H > -H ? m3 - H : -H, hi = m3 + H < H ? m3 + H : H;
-      const float4 bv = rb[(m3 + H) * kLanes + lane];
+    const float4* ra = rows + b * kRows + (kb * HB + 2 * BK - 1) * kLanes + lane;
+    const float4* rb = rows + b * kRows + kRow + lane;
+    // weights of square (kb, c): inside block (kb / per, c / per)
+    const int kB = kb / per;
+    const float* W0 = Wb + (2 * b) * PW + (sum_first_block(kB) - max(0, kB - 2)) * BK * BK + (kb % per) * HB;
+    auto wat = [&](int c) { return W0 + (c / per) * BK * BK + (c % per) * HB * BK; };
+    float4 win[HB];
+    int c = max(0, kb - D + 1);
+    if (kb >= D) {
+      const int cl = kb - D;
+      const float* w = wat(cl);
+      sum_block_df<-1, BK, HB>(w, w + PW, ra - cl * HB * kLanes, rb + cl * HB * kLanes, win, rh, rl, ih, il);
+    } else {
 #pragma unroll
-      for (int j = 0; j < NJ; j++) {
-        const int k3 = -H + warp + KW * j;
-        if (k3 >= lo && k3 <= hi) {
-          const int p = off + k3 - lo;
-          const float wh = Wh[p], wl = Wl[p];
-          const float4 av = ra[(k3 - m3 + H) * kLanes + lane];
-          // w b = (w b_re, w b_im), leading parts exact
-          float brh = wh * bv.x, brl = fmaf(wh, bv.x, -brh);
-          brl = fmaf(wh, bv.y, brl);
-          brl = fmaf(wl, bv.x, brl);
-          float bih = wh * bv.z, bil = fmaf(wh, bv.z, -bih);
-          bil = fmaf(wh, bv.w, bil);
-          bil = fmaf(wl, bv.z, bil);
-          // a (w b): re += a_re br - a_im bi, im += a_re bi + a_im br
-          df_mul_acc(av.x, av.y, brh, brl, rh[j], rl[j]);
-          df_mul_acc(-av.z, -av.w, bih, bil, rh[j], rl[j]);
-          df_mul_acc(av.x, av.y, bih, bil, ih[j], il[j]);
-          df_mul_acc(av.z, av.w, brh, brl, ih[j], il[j]);
-        }
-      }
-      off += hi - lo + 1;
+      for (int i = 1; i < HB; i++) win[i] = ra[i * kLanes];
+    }
+    const int c1 = min(NB - 1, kb + D - 1);
+#pragma unroll 1
+    for (; c <= c1; c++) {
+      const float* w = wat(c);
+      sum_block_df<0, BK, HB>(w, w + PW, ra - c * HB * kLanes, rb + c * HB * kLanes, win, rh, rl, ih, il);
+    }
+    if (kb < NB - D) {
+      const float* w = wat(c);
+      sum_block_df<1, BK, HB>(w, w + PW, ra, rb + c * HB * kLanes, win, rh, rl, ih, il);
     }
   }
   if (s_err) {
@@ -562,13 +650,12 @@ __global__ void __launch_bounds__(KW * 32, 2) k_sum_df(SumDfArgs a) {
     }
     return;
   }
-  double2* out = a.partial + ((long long)blockIdx.x * a.Gs + g) * n * kLanes;
+  double2* out = a.partial + ((long long)blockIdx.x * a.Gs + g) * kRow;
 #pragma unroll
-  for (int j = 0; j < NJ; j++) {
-    const int k3 = -H + warp + KW * j;
-    if (k3 <= H)
-      out[(k3 + H) * kLanes + lane] = make_double2((double)rh[j] + (double)rl[j], (double)ih[j] + (double)il[j]);
-  }
+  for (int i = 0; i < HB; i++)
+    if (kb * HB + i < n)
+      out[(kb * HB + i) * kLanes + lane] =
+          make_double2((double)rh[i] + (double)rl[i], (double)ih[i] + (double)il[i]);
 }
 
 // In place: every complex FP64 value of the transformed rows becomes its (hi, lo) float pairs
@@ -885,8 +972,8 @@ __global__ void __launch_bounds__(256) k_collide_bgk(const double* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------------------
-// Setup: weight blocks W[step][p] = beta_s for the (m3, k3) pairs of each (k1, k2, m1, m2)
-// step, in the loop order of k_sum, from the tables G[a2][b2] and Lo[m2] = G(2|m|, 0).
+// Setup: weights W[step][p] = beta_s of the (k3, m3) pairs of each (k1, k2, m1, m2) step, in the
+// block order of k_sum, from the tables G[a2][b2] and Lo[m2] = G(2|m|, 0).
 // ---------------------------------------------------------------------------------------
 template <typename T, bool LO>
 __global__ void k_build_weights(const int4* units, const long long* unit_step0, int n_units, int H, int PW,
@@ -898,25 +985,20 @@ __global__ void k_build_weights(const int4* units, const long long* unit_step0, 
   int m2lo = max(-H, k2 - H), m2hi = min(H, k2 + H);
   int nm2 = m2hi - m2lo + 1;
   int S = (ud.w - ud.z + 1) * nm2;
-  int np = 3 * H * H + 3 * H + 1;
+  const int BK = (H + 1) / 2, n = 2 * H + 1, np = sum_weights(BK);
   for (int s = blockIdx.y; s < S; s += gridDim.y) {
     int m1 = ud.z + s / nm2, m2 = m2lo + s % nm2;
     T* out = W + (unit_step0[u] + s) * PW;
     for (int p = threadIdx.x; p < PW; p += blockDim.x) {
-      if (p >= np) {
+      // p -> block (kb, c), m3, k3 in the k_sum order
+      const int blk = p / (BK * BK), in = p % (BK * BK);
+      const int kb = blk < 3 ? 0 : (blk < 7 ? 1 : (blk < 11 ? 2 : 3));
+      const int c = max(0, kb - 2) + blk - sum_first_block(kb);
+      const int ki = kb * BK + in % BK, mi = c * BK + in / BK;
+      const int k3 = ki - H, m3 = mi - H;
+      if (p >= np || ki >= n || mi >= n || abs(k3 - m3) > H) {
         out[p] = (T)0;
         continue;
-      }
-      // invert p -> (m3, k3) in the k_sum loop order
-      int q = p, m3 = -H, k3 = 0;
-      for (m3 = -H; m3 <= H; m3++) {
-        int lo = max(-H, m3 - H), hi = min(H, m3 + H);
-        int cnt = hi - lo + 1;
-        if (q < cnt) {
-          k3 = lo + q;
-          break;
-        }
-        q -= cnt;
       }
       long long a2 = (long long)k1 * k1 + (long long)k2 * k2 + (long long)k3 * k3;
       long long d1 = k1 - 2 * m1, d2 = k2 - 2 * m2, d3 = k3 - 2 * m3;
@@ -942,24 +1024,44 @@ static size_t dft_smem(int N, int extra_cplx, int extra_real) {
   return 2 * n * N * sizeof(T) + extra_cplx * sizeof(CT) + extra_real * sizeof(T);
 }
 
-template <typename T, int H>
-static cudaError_t launch_sum_t(const SumArgs<T>& a, int NW, int n_units, cudaStream_t st) {
+template <typename T, int BK, int F>
+static cudaError_t launch_sum_f(const SumArgs<T>& a, int NW, int n_units, cudaStream_t st) {
   typedef typename CplxOf<T>::type CT;
-  constexpr int n = 2 * H + 1;
-  constexpr int NP = 3 * H * H + 3 * H + 1;
+  constexpr int n = 4 * BK - 1;
   constexpr int VEC = 16 / (int)sizeof(T);
-  constexpr int PW = (NP + VEC - 1) / VEC * VEC;
-  constexpr int kRowBufs = sizeof(T) == 4 ? 1 : 2;
-  size_t smem = 2 * PW * sizeof(T) + (size_t)kRowBufs * NW * 2 * n * kLanes * sizeof(CT);
-  cudaError_t e = func_attr((const void*)k_sum<T, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int PWS = (sum_weights(BK) + VEC - 1) / VEC * VEC + (F > 1 ? VEC : 0);
+  // lane groups per block: as many as asked for, within an SM's shared memory
+  constexpr size_t wbytes = 2 * F * PWS * sizeof(T), gbytes = (size_t)2 * (2 * n + 1) * kLanes * sizeof(CT);
+  const int groups = a.G - a.g0;
+  const int NG = std::max(1, std::min(std::min(NW, groups), (int)((220 * 1024 - wbytes) / gbytes)));
+  const size_t smem = wbytes + NG * gbytes;
+  cudaError_t e = func_attr((const void*)k_sum<T, BK, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  dim3 grid(n_units, (a.G + NW - 1) / NW);
-  k_sum<T, H><<<grid, NW * 32, smem, st>>>(a);
+  dim3 grid(n_units, (groups + NG - 1) / NG);
+  k_sum<T, BK, F><<<grid, NG * 128, smem, st>>>(a);
   return cudaGetLastError();
 }
 
+template <typename T, int BK>
+static cudaError_t launch_sum_t(const SumArgs<T>& a, int NW, int n_units, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8) {
+    if (a.fold > 1) {  // the last group's rows hold 32 / fold lanes; the others are as usual
+      SumArgs<T> x = a;
+      if (a.G > 1) {
+        x.G = a.G - 1;
+        cudaError_t e = launch_sum_f<T, BK, 1>(x, NW, n_units, st);
+        if (e != cudaSuccess) return e;
+        x.G = a.G;
+      }
+      x.g0 = a.G - 1;
+      return a.fold == 4 ? launch_sum_f<T, BK, 4>(x, 1, n_units, st) : launch_sum_f<T, BK, 2>(x, 1, n_units, st);
+    }
+  }
+  return launch_sum_f<T, BK, 1>(a, NW, n_units, st);
+}
+
 int sum_pad(int H, int elem_bytes) {
-  int NP = 3 * H * H + 3 * H + 1, VEC = 16 / elem_bytes;
+  int NP = sum_weights((H + 1) / 2), VEC = 16 / elem_bytes;
   return (NP + VEC - 1) / VEC * VEC;
 }
 
@@ -967,39 +1069,37 @@ template <typename T>
 cudaError_t launch_sum(const SumArgs<T>& a, int H, int NW, int n_units, cudaStream_t st) {
   if (NW < 1 || NW > 4) return cudaErrorInvalidValue;
   switch (H) {
-    case 3: return launch_sum_t<T, 3>(a, NW, n_units, st);
-    case 5: return launch_sum_t<T, 5>(a, NW, n_units, st);
-    case 7: return launch_sum_t<T, 7>(a, NW, n_units, st);
-    case 9: return launch_sum_t<T, 9>(a, NW, n_units, st);
-    case 11: return launch_sum_t<T, 11>(a, NW, n_units, st);
-    case 13: return launch_sum_t<T, 13>(a, NW, n_units, st);
-    case 15: return launch_sum_t<T, 15>(a, NW, n_units, st);
+    case 3: return launch_sum_t<T, 2>(a, NW, n_units, st);
+    case 5: return launch_sum_t<T, 3>(a, NW, n_units, st);
+    case 7: return launch_sum_t<T, 4>(a, NW, n_units, st);
+    case 9: return launch_sum_t<T, 5>(a, NW, n_units, st);
+    case 11: return launch_sum_t<T, 6>(a, NW, n_units, st);
+    case 13: return launch_sum_t<T, 7>(a, NW, n_units, st);
+    case 15: return launch_sum_t<T, 8>(a, NW, n_units, st);
   }
   return cudaErrorInvalidValue;
 }
 
-template <int H>
+template <int BK>
 static cudaError_t launch_sum_df_t(const SumDfArgs& a, int n_units, cudaStream_t st) {
-  constexpr int n = 2 * H + 1;
-  constexpr int NP = 3 * H * H + 3 * H + 1;
-  constexpr int PW = (NP + 3) / 4 * 4;
-  constexpr int KW = H >= 7 ? 8 : 4;
-  size_t smem = 4 * PW * sizeof(float) + 4 * (size_t)n * kLanes * sizeof(float4);
-  cudaError_t e = func_attr((const void*)k_sum_df<H, KW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int n = 4 * BK - 1;
+  constexpr int PW = (sum_weights(BK) + 3) / 4 * 4;
+  const size_t smem = 4 * PW * sizeof(float) + (size_t)2 * (2 * n + 1) * kLanes * sizeof(float4);
+  cudaError_t e = func_attr((const void*)k_sum_df<BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_sum_df<H, KW><<<dim3(n_units, a.G), KW * 32, smem, st>>>(a);
+  k_sum_df<BK><<<dim3(n_units, a.G), 128 * (BK / df_side(BK)), smem, st>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sum_df(const SumDfArgs& a, int H, int n_units, cudaStream_t st) {
   switch (H) {
-    case 3: return launch_sum_df_t<3>(a, n_units, st);
-    case 5: return launch_sum_df_t<5>(a, n_units, st);
-    case 7: return launch_sum_df_t<7>(a, n_units, st);
-    case 9: return launch_sum_df_t<9>(a, n_units, st);
-    case 11: return launch_sum_df_t<11>(a, n_units, st);
-    case 13: return launch_sum_df_t<13>(a, n_units, st);
-    case 15: return launch_sum_df_t<15>(a, n_units, st);
+    case 3: return launch_sum_df_t<2>(a, n_units, st);
+    case 5: return launch_sum_df_t<3>(a, n_units, st);
+    case 7: return launch_sum_df_t<4>(a, n_units, st);
+    case 9: return launch_sum_df_t<5>(a, n_units, st);
+    case 11: return launch_sum_df_t<6>(a, n_units, st);
+    case 13: return launch_sum_df_t<7>(a, n_units, st);
+    case 15: return launch_sum_df_t<8>(a, n_units, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -59,6 +59,8 @@ struct SpecBufs {
   CT *st1a, *st1b;       // [C][N][N][n]
   CT *st2a, *st2b;       // [C][N][n][n]
   CT *ahat, *bhat;       // [G][n][n][n][32]
+  // one group (-1: none) whose rows hold fewer lanes, [n][n][n][fold_lanes] at the same place (FP64)
+  int fold_group = -1, fold_lanes = kLanes;
   CT* qhat;              // [G][n][n][n][32]
   const int* cell_inst;  // instance of each cell, and the per-instance activity (nullable):
   const int* active;     // the transforms skip the cells of converged instances
@@ -74,6 +76,8 @@ struct SumArgs {
   const CT* bhat;
   CT* partial;                  // [units][Gs][n][32]
   int G;                        // groups of this launch (ahat, bhat, partial start at its first group)
+  int g0 = 0;                   // first of them to compute
+  int fold = 1;                 // FP64: steps that a warp takes at once in the last group (2, 4)
   int Gs;                       // group stride of partial (the handle's group count)
   Counters* cnt;
   long long spin_max;

@@ -604,6 +604,14 @@ CollideCtx<T> collide_ctx(const sgs_handle* h, int l = 0, int g_lo = 0, int g_hi
   x.sum.bhat = x.sb.bhat;
   x.sum.partial = h->at<CT>(h->off.partial) + (size_t)g_lo * n * kLanes;
   x.sum.G = g_hi - g_lo;
+  // FP64 sum: a last lane group of at most 16 or 8 cells takes 2 or 4 steps at once (the
+  // double-float sum reads the usual layout: collide_impl undoes this)
+  const int last = x.C - (x.sum.G - 1) * kLanes;
+  if (sizeof(T) == 8 && last <= kLanes / 2) {
+    x.sum.fold = last <= kLanes / 4 ? 4 : 2;
+    x.sb.fold_group = x.sum.G - 1;
+    x.sb.fold_lanes = kLanes / x.sum.fold;
+  }
   x.sum.Gs = Gl;
   x.sum.cnt = h->at<Counters>(h->off.cnt);
   x.sum.spin_max = h->spin_max;
@@ -707,6 +715,8 @@ int collide_impl(sgs_handle* h, const double* f, double* Q, double* P, int preci
   if (precision == SGS_DF64) {
     if (h->precision != SGS_FP32) return SGS_ERR_ARG;  // FP32 tables not built
     CollideCtx<double> x = collide_ctx<double>(h, l, g_lo, g_hi);
+    x.sum.fold = 1;
+    x.sb.fold_group = -1;
     cudaError_t er;
     {
       Scope sc(h, SGS_PROF_DFT, st, 6);
