@@ -21,22 +21,160 @@
 
 namespace sgs {
 
+// Factor d of the Maxwellian with exponents th at node i (the first one carries exp(alpha)).
+__device__ inline double maxwell_factor(const double* th, int d, int i, int N, double dv) {
+  const double v = node(i, N, dv);
+  double x = th[1 + d] * v - th[4] * v * v;
+  if (d == 0) x += th[0];
+  return exp(x);
+}
+
 // ---------------------------------------------------------------------------------------
-// Moments and discrete Maxwellian of every cell.
+// Discrete Maxwellian on the tensor grid (eqs. (13)-(14)).
+//
+// M_k = exp(alpha + beta.v_k - gamma |v_k|^2) factorises as
+//   exp(alpha) * E_1(v_1) E_2(v_2) E_3(v_3),   E_d(v) = exp(beta_d v - gamma v^2),
+// so every moment sum_k w phi_i phi_j M_k with phi = (1, v1, v2, v3, |v|^2) is a product of
+// one-dimensional sums S_d^p = sum_i E_d(v_i) v_i^p, p = 0..4, and a Newton iteration costs O(N)
+// instead of O(N^3). The iteration itself (undamped Newton with step halving while the scaled
+// residual grows; stop one step after the exponent change |da| + L sum|db| + L^2 |dg| falls below
+// tol) follows the discrete conservation equations directly.
+//
+// Called by one full warp; lane i < N handles node i. All lanes return the same result. The 15
+// sums are reduced together: a lane keeps half of its values in each step and hands the other
+// half to its partner (16 additions instead of 75 of the scarce FP64 pipe, the same pairs).
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_moments(const double* __restrict__ f, CellTables ct, int N, double dv,
-                                                  double newton_tol, int newton_max, double* __restrict__ theta,
-                                                  double* __restrict__ nu, Counters* cnt) {
+struct MaxwEval {
+  double F[5];  // moments of M minus the target
+  float A[15];  // upper triangle of sum w M phi phi^T (row-major, i <= j): Newton direction only
+  double fn;    // max |F_i| / |target_0|
+};
+
+__device__ inline void maxw_eval(int N, double dv, double w, const double* target, const double* th, MaxwEval& out) {
+  const int lane = threadIdx.x & 31;
+  double v[16];
+  const double vd = node(lane < N ? lane : 0, N, dv), v2 = vd * vd;
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    const double x = lane < N ? exp(th[1 + d] * vd - th[4] * vd * vd) : 0.0;
+    v[5 * d + 0] = x;
+    v[5 * d + 1] = x * vd;
+    v[5 * d + 2] = v[5 * d + 1] * vd;
+    v[5 * d + 3] = v[5 * d + 2] * vd;
+    v[5 * d + 4] = v[5 * d + 2] * v2;
+  }
+  v[15] = 0.0;
+  int o = 16;
+#pragma unroll
+  for (int h = 8; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int q = 0; q < h; q++) {
+      const double send = up ? v[q] : v[q + h], keep = up ? v[q + h] : v[q];
+      v[q] = keep + shfl_x(send, o);
+    }
+  }
+  const double t = v[0] + shfl_x(v[0], 1);  // total of value lane / 2
+  const float tf = (float)t;
+  double s[15];
+  float f[15];
+#pragma unroll
+  for (int q = 0; q < 15; q++) {
+    s[q] = __shfl_sync(0xffffffffu, t, 2 * q);
+    f[q] = __shfl_sync(0xffffffffu, tf, 2 * q);
+  }
+  const double ea = exp(th[0]);
+  const double *S1 = s, *S2 = s + 5, *S3 = s + 10;
+  const double c = w * ea;
+  // sums of phi_i M over the grid, from the 1-D sums
+  const double s23 = S2[0] * S3[0];
+  const double mom[5] = {S1[0] * s23, S1[1] * s23, S1[0] * (S2[1] * S3[0]), S1[0] * (S2[0] * S3[1]),
+                         S1[2] * s23 + S1[0] * (S2[2] * S3[0] + S2[0] * S3[2])};
+  double amax = 0.0;
+#pragma unroll
+  for (int i = 0; i < 5; i++) {
+    out.F[i] = c * mom[i] - target[i];
+    amax = fmax(amax, fabs(out.F[i]));
+  }
+  out.fn = amax / fabs(target[0]);
+  // Jacobian entries in FP32: they only set the Newton direction
+  const float *f1 = f, *f2 = f + 5, *f3 = f + 10;
+  float q11 = f1[2] * f2[0] * f3[0], q22 = f1[0] * f2[2] * f3[0], q33 = f1[0] * f2[0] * f3[2];
+  float q12 = f1[1] * f2[1] * f3[0], q13 = f1[1] * f2[0] * f3[1], q23 = f1[0] * f2[1] * f3[1];
+  float c1 = f1[3] * f2[0] * f3[0] + f1[1] * f2[2] * f3[0] + f1[1] * f2[0] * f3[2];
+  float c2 = f1[2] * f2[1] * f3[0] + f1[0] * f2[3] * f3[0] + f1[0] * f2[1] * f3[2];
+  float c3 = f1[2] * f2[0] * f3[1] + f1[0] * f2[2] * f3[1] + f1[0] * f2[0] * f3[3];
+  float e4 = f1[4] * f2[0] * f3[0] + f1[0] * f2[4] * f3[0] + f1[0] * f2[0] * f3[4] +
+             2.0f * (f1[2] * f2[2] * f3[0] + f1[2] * f2[0] * f3[2] + f1[0] * f2[2] * f3[2]);
+  float cf = (float)c;
+  float A[15] = {f1[0] * f2[0] * f3[0], f1[1] * f2[0] * f3[0], f1[0] * f2[1] * f3[0], f1[0] * f2[0] * f3[1],
+                 q11 + q22 + q33, q11, q12, q13, c1, q22, q23, c2, q33, c3, e4};
+#pragma unroll
+  for (int i = 0; i < 15; i++) out.A[i] = cf * A[i];
+}
+
+// Newton for the discrete Maxwellian from the guess in th. The residual F is evaluated in FP64 and
+// the direction from the FP32 factorisation (inexact Newton: the root is the one of F). The step
+// is halved while the scaled residual grows; the iteration stops right after a step whose
+// exponent change |da| + L sum|db| + L^2 |dg| is below tol.
+__device__ inline int maxwellian_newton(int N, double dv, double w, const double* target, double* th, double tol,
+                                        int maxit) {
+  const double L = node(N - 1, N, dv);
+  MaxwEval ev;
+  maxw_eval(N, dv, w, target, th, ev);
+  for (int it = 0; it < maxit; it++) {
+    float y[5], Ff[5];
+#pragma unroll
+    for (int i = 0; i < 5; i++) Ff[i] = (float)ev.F[i];
+    if (!chol5_solve(ev.A, Ff, y)) return -1;
+    double d[5] = {-(double)y[0], -(double)y[1], -(double)y[2], -(double)y[3], (double)y[4]};  // -D A^{-1} F
+    double lam = 1.0;
+    double fn = ev.fn;
+    double tt[5];
+    for (int hv = 0; hv < 40; hv++) {
+#pragma unroll
+      for (int i = 0; i < 5; i++) tt[i] = th[i] + lam * d[i];
+      maxw_eval(N, dv, w, target, tt, ev);
+      if (ev.fn == ev.fn && (ev.fn <= fn || ev.fn <= 1e-10)) break;
+      lam *= 0.5;
+    }
+#pragma unroll
+    for (int i = 0; i < 5; i++) th[i] = tt[i];
+    double step = lam * (fabs(d[0]) + L * (fabs(d[1]) + fabs(d[2]) + fabs(d[3])) + L * L * fabs(d[4]));
+    if (!(step == step)) return -1;
+    if (step <= tol) return it + 1;
+  }
+  return -1;
+}
+
+// ---------------------------------------------------------------------------------------
+// Moments and discrete Maxwellian of every cell, its collision frequency and the separable
+// factors of the Maxwellian (E_d[i], E_1 with exp(alpha)) that the transforms read.
+//
+// The sums are bound by the FP64 pipe of one SM (8 instructions a node: 85 us for 32^3 nodes). For
+// a call of few cells the eight warps of a cell are therefore eight CTAs of a cluster (SPLIT), on
+// as many SMs; every warp adds the same nodes in the same order in both forms, so the results
+// are the same bits. 32 cells of 32^3: 132 -> 89 us, 8 cells of 8^3: 57 -> 44 us (the rest is
+// Newton, on one warp: an FP64 instruction takes a scheduler 64 cycles, in a chain or not).
+// ---------------------------------------------------------------------------------------
+template <bool SPLIT>
+__global__ void __launch_bounds__(SPLIT ? 32 : 256) k_moments(const double* __restrict__ f, CellTables ct, int N,
+                                                               double dv, double newton_tol, int newton_max,
+                                                               double* __restrict__ theta, double* __restrict__ nu,
+                                                               double* __restrict__ efac, Counters* cnt) {
   __shared__ double vv[kMaxN];
   __shared__ double part[8][5];
-  int c = blockIdx.x;
-  if (!cell_active(ct.active, ct.cell_inst, c)) return;
+  const int wid = SPLIT ? (int)(blockIdx.x & 7) : (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int c = SPLIT ? blockIdx.x >> 3 : blockIdx.x;
+  if (!cell_active(ct.active, ct.cell_inst, c)) return;  // whole cluster, uniformly
   int K = N * N * N;
   const double* fc = f + ct.cell_off[c];
   if (threadIdx.x < N) vv[threadIdx.x] = node(threadIdx.x, N, dv);
+  if (SPLIT) cg::this_cluster().barrier_arrive();  // (every CTA runs before another writes into it)
   __syncthreads();
   double s[5] = {0, 0, 0, 0, 0};
-  for (int e = threadIdx.x; e < K; e += blockDim.x) {
+#pragma unroll 4
+  for (int e = wid * 32 + lane; e < K; e += 256) {
     int i3 = e % N, i2 = (e / N) % N, i1 = e / (N * N);
     double x = fc[e];
     double a = vv[i1], b = vv[i2], d = vv[i3];
@@ -47,24 +185,32 @@ __global__ void __launch_bounds__(256) k_moments(const double* __restrict__ f, C
     s[4] += x * (a * a + b * b + d * d);
   }
   warp_allsum<5>(s);
-  int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0)
-    for (int q = 0; q < 5; q++) part[wid][q] = s[q];
-  __syncthreads();
-  if (wid != 0) return;
+  if (SPLIT) {
+    cg::cluster_group cl = cg::this_cluster();
+    cl.barrier_wait();
+    if (lane == 0) {
+      double* p = cl.map_shared_rank(&part[wid][0], 0);  // rank = wid: a cluster is one cell
+      for (int q = 0; q < 5; q++) p[q] = s[q];
+    }
+    cl.sync();
+    if (wid != 0) return;  // only its own writes were remote, and they have landed
+  } else {
+    if (lane == 0)
+      for (int q = 0; q < 5; q++) part[wid][q] = s[q];
+    __syncthreads();
+    if (wid != 0) return;
+  }
   double w = dv * dv * dv;
   double m[5];
   for (int q = 0; q < 5; q++) {
     double t = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); k++) t += part[k][q];
+    for (int k = 0; k < 8; k++) t += part[k][q];
     m[q] = w * t;
   }
   const InstDev& I = ct.inst[ct.cell_inst[c]];
   double th[5] = {0, 0, 0, 0, 0};
-  MaxwEval<double> ev;
   int it = -1;
-  if (continuum_guess<double>(m, th))
-    it = maxwellian_newton<double>(N, dv, w, false, 0.0, m, th, newton_tol, newton_max, ev);
+  if (continuum_guess<double>(m, th)) it = maxwellian_newton(N, dv, w, m, th, newton_tol, newton_max);
   double rho = m[0];
   double T = (m[4] / rho - (m[1] * m[1] + m[2] * m[2] + m[3] * m[3]) / (rho * rho)) / 3.0;
   // penalty frequency of eq. (28): the loss frequency 4 pi b0 rho for Maxwell molecules;
@@ -82,25 +228,16 @@ __global__ void __launch_bounds__(256) k_moments(const double* __restrict__ f, C
     if (!(rho == rho) || !(T == T)) bits |= SGS_ST_NONFINITE;
     if (bits) atomicOr(&cnt[ct.cell_inst[c]].status, bits);
   }
+  for (int d = 0; d < 3; d++)
+    if (lane < N) efac[((long long)c * 3 + d) * kMaxN + lane] = maxwell_factor(th, d, lane, N, dv);
 }
 
-// Per-block factors E_d[i] of the discrete Maxwellian of cell c (E_1 carries exp(alpha)).
-__device__ inline void maxwell_factors(const double* theta, int c, int N, double dv, double* E /*[3][kMaxN]*/);
-
-// Separable factors of every cell's Maxwellian, once per collision step (one block per
-// cell), for the transform passes to read instead of re-evaluating 3N exponentials per block.
+// Separable factors of every cell's Maxwellian from theta (one block per cell): of a reference
+// state, whose moments are not formed.
 __global__ void k_factors(const double* theta, int N, double dv, double* efac) {
-  maxwell_factors(theta, blockIdx.x, N, dv, efac + (long long)blockIdx.x * 3 * kMaxN);
-}
-
-__device__ inline void maxwell_factors(const double* theta, int c, int N, double dv, double* E /*[3][kMaxN]*/) {
   if (threadIdx.x < 3 * N) {
-    int d = threadIdx.x / N, i = threadIdx.x % N;
-    const double* th = theta + 5 * c;
-    double v = node(i, N, dv);
-    double x = th[1 + d] * v - th[4] * v * v;
-    if (d == 0) x += th[0];
-    E[d * kMaxN + i] = exp(x);
+    const int d = threadIdx.x / N, i = threadIdx.x % N;
+    efac[((long long)blockIdx.x * 3 + d) * kMaxN + i] = maxwell_factor(theta + 5 * (long long)blockIdx.x, d, i, N, dv);
   }
 }
 
@@ -959,7 +1096,10 @@ __global__ void __launch_bounds__(256) k_collide_bgk(const double* __restrict__ 
   __shared__ double E[3 * kMaxN];
   int c = blockIdx.x, i1 = blockIdx.y;
   if (!cell_active(ct.active, ct.cell_inst, c)) return;
-  maxwell_factors(theta, c, N, dv, E);
+  if (threadIdx.x < 3 * N) {
+    const int d = threadIdx.x / N, i = threadIdx.x % N;
+    E[d * kMaxN + i] = maxwell_factor(theta + 5 * (long long)c, d, i, N, dv);
+  }
   __syncthreads();
   long long base = ct.cell_off[c] + (long long)i1 * N * N;
   double nuc = nu[c];
@@ -1113,8 +1253,9 @@ template <typename T>
 cudaError_t launch_dft(const double* f, const CollideCtx<T>& x, const DftMode& md, cudaStream_t st) {
   int N = x.N, n = N - 1, C = x.C;
   cudaError_t e;
-  k_factors<<<C, 3 * N, 0, st>>>(x.theta, N, x.dv, x.efac);
-  if (md.mode != 0) k_factors<<<C, 3 * N, 0, st>>>(md.theta_ref, N, x.dv, x.efac_ref);
+  // the factors of this step were written by launch_moments, those of the reference by the first
+  // of the two transforms of an increment
+  if (md.mode == 1) k_factors<<<C, 3 * N, 0, st>>>(md.theta_ref, N, x.dv, x.efac_ref);
   size_t sm1 = dft_smem<T>(N, 0, 2 * N * N);
   e = func_attr((const void*)k_dft_i3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
   if (e != cudaSuccess) return e;
@@ -1171,10 +1312,29 @@ cudaError_t launch_factors(const double* theta, int C, int N, double dv, double*
   return cudaGetLastError();
 }
 
+// Cells below which the warps of a cell go to different SMs: with more of them the chip's FP64
+// pipes are busy either way, and a CTA per warp only adds launches (128 cells of 32^3: 132 us in
+// one CTA a cell, 122 split).
+constexpr int kMomentsSplit = 304;
+
 cudaError_t launch_moments(const double* f, const CellTables& ct, int C, int N, double dv, double tol, int maxit,
-                           double* theta, double* nu, Counters* cnt, cudaStream_t st) {
-  k_moments<<<C, 256, 0, st>>>(f, ct, N, dv, tol, maxit, theta, nu, cnt);
-  return cudaGetLastError();
+                           double* theta, double* nu, double* efac, Counters* cnt, cudaStream_t st) {
+  if (C > kMomentsSplit) {
+    k_moments<false><<<C, 256, 0, st>>>(f, ct, N, dv, tol, maxit, theta, nu, efac, cnt);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(8 * C);
+  cfg.blockDim = dim3(32);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 8;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_moments<true>, f, ct, N, dv, tol, maxit, theta, nu, efac, cnt);
 }
 
 cudaError_t launch_collide_bgk(const double* f, const CellTables& ct, int C, int N, double dv, const double* theta,

@@ -167,16 +167,6 @@ __device__ __forceinline__ double exp_in(double x) { return exp(x); }
 __device__ __forceinline__ float exp_in(float x) { return expf(x); }
 __device__ __forceinline__ dfloat exp_in(dfloat x) { return df_exp(x); }
 
-// exp evaluated in FP64 for double and df64, in FP32 for float
-template <typename E>
-__device__ __forceinline__ E exp_e(double x) {
-  return cvt<E>(exp(x));
-}
-template <>
-__device__ __forceinline__ float exp_e<float>(double x) {
-  return expf((float)x);
-}
-
 __device__ __forceinline__ double shfl_x(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ float shfl_x(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ dfloat shfl_x(dfloat v, int o) {
@@ -193,89 +183,6 @@ __device__ inline void warp_allsum(T (&x)[NV]) {
 #pragma unroll
     for (int q = 0; q < NV; q++) x[q] += shfl_x(x[q], o);
   }
-}
-
-// ---------------------------------------------------------------------------------------
-// Discrete Maxwellian on the tensor grid (eqs. (13)-(14)).
-//
-// M_k = exp(alpha + beta.v_k - gamma |v_k|^2) factorises as
-//   exp(alpha) * E_1(v_1) E_2(v_2) E_3(v_3),   E_d(v) = exp(beta_d v - gamma v^2),
-// and so do the weights used here (w, or w |v1|/dx for step 1 of PFP, eq. (24)). Every
-// weighted moment sum_k wk phi_i phi_j M_k with phi = (1, v1, v2, v3, |v|^2) is therefore a
-// product of one-dimensional sums S_d^p = sum_i omega_d(v_i) E_d(v_i) v_i^p, p = 0..4, and a
-// Newton iteration costs O(N) instead of O(N^3). The iteration itself (undamped Newton
-// with step halving while the scaled residual grows; stop one step after the exponent
-// change |da| + L sum|db| + L^2 |dg| falls below tol) follows the discrete conservation
-// equations directly.
-//
-// Called by one full warp; lane i < N handles node i. All lanes return the same result.
-// ---------------------------------------------------------------------------------------
-template <typename E>
-struct MaxwEval {
-  E F[5];        // weighted moments of M minus the target
-  float A[15];   // upper triangle of sum wk M phi phi^T (row-major, i <= j): Newton direction only
-  double fn;     // max |F_i| / |target_0|
-  E e[3];        // this lane's E_1 (with exp(alpha)), E_2, E_3
-};
-
-template <typename E>
-__device__ inline void maxw_eval(int N, double dv, double w, bool wv1, double inv_dx, const E* target,
-                                 const double* th, MaxwEval<E>& out) {
-  int lane = threadIdx.x & 31;
-  E s[15];
-  double vd = node(lane < N ? lane : 0, N, dv);
-  E vi = cvt<E>(vd), v2 = cvt<E>(vd * vd);
-#pragma unroll
-  for (int d = 0; d < 3; d++) {
-    E e = lane < N ? exp_e<E>(th[1 + d] * vd - th[4] * vd * vd) : cvt<E>(0.0);
-    out.e[d] = e;
-    E x = (d == 0 && wv1) ? cvt<E>(fabs(vd) * inv_dx) * e : e;
-    s[5 * d + 0] = x;
-    s[5 * d + 1] = x * vi;
-    s[5 * d + 2] = s[5 * d + 1] * vi;
-    s[5 * d + 3] = s[5 * d + 2] * vi;
-    s[5 * d + 4] = s[5 * d + 2] * v2;
-  }
-  warp_allsum<15, E>(s);
-  E ea = exp_e<E>(th[0]);
-  out.e[0] = out.e[0] * ea;
-  const E* S1 = s;
-  const E* S2 = s + 5;
-  const E* S3 = s + 10;
-  E c = cvt<E>(w) * ea;
-  // sums of phi_i M over the grid, from the 1-D sums
-  E s23 = S2[0] * S3[0];
-  E m00 = S1[0] * s23;
-  E m1 = S1[1] * s23, m2 = S1[0] * (S2[1] * S3[0]), m3 = S1[0] * (S2[0] * S3[1]);
-  E e2 = S1[2] * s23 + S1[0] * (S2[2] * S3[0] + S2[0] * S3[2]);
-  E mom[5] = {m00, m1, m2, m3, e2};
-  double amax = 0.0;
-#pragma unroll
-  for (int i = 0; i < 5; i++) {
-    out.F[i] = c * mom[i] - target[i];
-    amax = fmax(amax, fabs(tod(out.F[i])));
-  }
-  out.fn = amax / fabs(tod(target[0]));
-  // Jacobian entries in FP32: they only set the Newton direction
-  float f1[5], f2[5], f3[5];
-#pragma unroll
-  for (int p = 0; p < 5; p++) {
-    f1[p] = (float)tod(S1[p]);
-    f2[p] = (float)tod(S2[p]);
-    f3[p] = (float)tod(S3[p]);
-  }
-  float q11 = f1[2] * f2[0] * f3[0], q22 = f1[0] * f2[2] * f3[0], q33 = f1[0] * f2[0] * f3[2];
-  float q12 = f1[1] * f2[1] * f3[0], q13 = f1[1] * f2[0] * f3[1], q23 = f1[0] * f2[1] * f3[1];
-  float c1 = f1[3] * f2[0] * f3[0] + f1[1] * f2[2] * f3[0] + f1[1] * f2[0] * f3[2];
-  float c2 = f1[2] * f2[1] * f3[0] + f1[0] * f2[3] * f3[0] + f1[0] * f2[1] * f3[2];
-  float c3 = f1[2] * f2[0] * f3[1] + f1[0] * f2[2] * f3[1] + f1[0] * f2[0] * f3[3];
-  float e4 = f1[4] * f2[0] * f3[0] + f1[0] * f2[4] * f3[0] + f1[0] * f2[0] * f3[4] +
-             2.0f * (f1[2] * f2[2] * f3[0] + f1[2] * f2[0] * f3[2] + f1[0] * f2[2] * f3[2]);
-  float cf = (float)tod(c);
-  float A[15] = {f1[0] * f2[0] * f3[0], f1[1] * f2[0] * f3[0], f1[0] * f2[1] * f3[0], f1[0] * f2[0] * f3[1],
-                 q11 + q22 + q33, q11, q12, q13, c1, q22, q23, c2, q33, c3, e4};
-#pragma unroll
-  for (int i = 0; i < 15; i++) out.A[i] = cf * A[i];
 }
 
 // Solves A y = b (FP32) for the symmetric positive definite 5x5 matrix given by its upper
@@ -357,41 +264,6 @@ __device__ inline bool continuum_guess(const E* m, double* th) {
   th[3] = U2 / T;
   th[0] = log(rho / (2.0 * kPi * T * sqrt(2.0 * kPi * T))) - 0.5 * uu / T;
   return true;
-}
-
-// Newton for the weighted discrete Maxwellian from the guess in th. The residual F is
-// evaluated in E (FP64 or FP32) and the direction from the FP32 factorisation (inexact
-// Newton: the root is the one of F in E). The step is halved while the scaled residual
-// grows; the iteration stops right after a step whose exponent change
-// |da| + L sum|db| + L^2 |dg| is below tol. On return ev holds the evaluation at th.
-template <typename E>
-__device__ inline int maxwellian_newton(int N, double dv, double w, bool wv1, double inv_dx, const E* target,
-                                        double* th, double tol, int maxit, MaxwEval<E>& ev) {
-  double L = node(N - 1, N, dv);
-  maxw_eval<E>(N, dv, w, wv1, inv_dx, target, th, ev);
-  for (int it = 0; it < maxit; it++) {
-    float y[5], Ff[5];
-#pragma unroll
-    for (int i = 0; i < 5; i++) Ff[i] = (float)tod(ev.F[i]);
-    if (!chol5_solve(ev.A, Ff, y)) return -1;
-    double d[5] = {-(double)y[0], -(double)y[1], -(double)y[2], -(double)y[3], (double)y[4]};  // -D A^{-1} F
-    double lam = 1.0;
-    double fn = ev.fn;
-    double tt[5];
-    for (int hv = 0; hv < 40; hv++) {
-#pragma unroll
-      for (int i = 0; i < 5; i++) tt[i] = th[i] + lam * d[i];
-      maxw_eval<E>(N, dv, w, wv1, inv_dx, target, tt, ev);
-      if (ev.fn == ev.fn && (ev.fn <= fn || ev.fn <= 1e-10)) break;
-      lam *= 0.5;
-    }
-#pragma unroll
-    for (int i = 0; i < 5; i++) th[i] = tt[i];
-    double step = lam * (fabs(d[0]) + L * (fabs(d[1]) + fabs(d[2]) + fabs(d[3])) + L * L * fabs(d[4]));
-    if (!(step == step)) return -1;
-    if (step <= tol) return it + 1;
-  }
-  return -1;
 }
 
 // ---------------------------------------------------------------------------------------

@@ -197,7 +197,7 @@ cudaError_t launch_slope_rhs2d(const AuxArgs& a, const double* f, const double* 
 cudaError_t launch_si_transport(const AuxArgs& a, double* f, const double* P, const double* rhs, const double* efac,
                                 const double* nu, cudaStream_t st);
 cudaError_t launch_moments(const double* f, const CellTables& ct, int C, int N, double dv, double tol, int maxit,
-                           double* theta, double* nu, Counters* cnt, cudaStream_t st);
+                           double* theta, double* nu, double* efac, Counters* cnt, cudaStream_t st);
 cudaError_t launch_collide_bgk(const double* f, const CellTables& ct, int C, int N, double dv, const double* theta,
                                const double* nu, double* Q, double* P, cudaStream_t st);
 template <typename T>

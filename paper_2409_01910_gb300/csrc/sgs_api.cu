@@ -653,7 +653,7 @@ int collide_impl(sgs_handle* h, const double* f, double* Q, double* P, int preci
   {
     Scope sc(h, SGS_PROF_MOMENTS, st, 1);
     e = launch_moments(f, ct, C, h->N, h->dv, p0.newton_tol, p0.newton_max, theta, nu,
-                       h->at<Counters>(h->off.cnt), st);
+                       h->at<double>(h->off.efac) + (size_t)3 * kMaxN * c0, h->at<Counters>(h->off.cnt), st);
   }
   if (e != cudaSuccess) return cuda_status(e);
   if (!h->spectral) {
@@ -663,7 +663,7 @@ int collide_impl(sgs_handle* h, const double* f, double* Q, double* P, int preci
   auto run = [&](auto x) -> int {
     cudaError_t er;
     {
-      Scope sc(h, SGS_PROF_DFT, st, 4);
+      Scope sc(h, SGS_PROF_DFT, st, 3);
       er = launch_dft(f, x, DftMode{0, nullptr, nullptr}, st);
     }
     if (er != cudaSuccess) return cuda_status(er);
@@ -686,7 +686,7 @@ int collide_impl(sgs_handle* h, const double* f, double* Q, double* P, int preci
     CT* part2 = h->at<CT>(h->off.partial2) + (size_t)g_lo * h->n * kLanes;
     cudaError_t er;
     {
-      Scope sc(h, SGS_PROF_DFT, st, 5);
+      Scope sc(h, SGS_PROF_DFT, st, 4);
       er = launch_dft(f, x, m1, st);
     }
     if (er != cudaSuccess) return cuda_status(er);
@@ -696,7 +696,7 @@ int collide_impl(sgs_handle* h, const double* f, double* Q, double* P, int preci
     }
     if (er != cudaSuccess) return cuda_status(er);
     {
-      Scope sc(h, SGS_PROF_DFT, st, 5);
+      Scope sc(h, SGS_PROF_DFT, st, 3);
       er = launch_dft(f, x, m2, st);
       if (er == cudaSuccess)
         er = cudaMemcpyAsync(x.sb.ahat, h->at<CT>(Lv.rah) + (size_t)g_lo * h->n * h->n * h->n * kLanes,
@@ -719,7 +719,7 @@ int collide_impl(sgs_handle* h, const double* f, double* Q, double* P, int preci
     x.sb.fold_group = -1;
     cudaError_t er;
     {
-      Scope sc(h, SGS_PROF_DFT, st, 6);
+      Scope sc(h, SGS_PROF_DFT, st, 5);
       er = launch_dft(f, x, DftMode{0, nullptr, nullptr}, st);
       const long long cnt = (long long)(g_hi - g_lo) * h->n * h->n * h->n * kLanes;
       if (er == cudaSuccess) er = launch_split_spec(x.sb.ahat, cnt, st);
@@ -1381,7 +1381,7 @@ int sgs_dc_step(sgs_handle* h, double* f, double* Q, double* P, int lo_iters, do
   if (e != cudaSuccess) return cuda_status(e);
   {
     CollideCtx<float> x = collide_ctx<float>(h);
-    Scope sc(h, SGS_PROF_DFT, st, 4);
+    Scope sc(h, SGS_PROF_DFT, st, 3);
     e = launch_dft(f, x, DftMode{0, nullptr, nullptr}, st);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(h->ws + h->off.ahat_ref, x.sb.ahat,
@@ -1824,11 +1824,11 @@ int sgs_fast_collide(sgs_fast* x, sgs_handle* h, const double* f, double* Q, int
     Scope sc(h, SGS_PROF_MOMENTS, st, 1);
     const sgs_problem& p0 = h->prob[0];
     e = launch_moments(f, cx.ct, h->C, h->N, h->dv, p0.newton_tol, p0.newton_max, h->at<double>(h->off.theta),
-                       h->at<double>(h->off.nu), h->at<Counters>(h->off.cnt), st);
+                       h->at<double>(h->off.nu), h->at<double>(h->off.efac), h->at<Counters>(h->off.cnt), st);
   }
   if (e != cudaSuccess) return cuda_status(e);
   {
-    Scope sc(h, SGS_PROF_DFT, st, 5);
+    Scope sc(h, SGS_PROF_DFT, st, 4);
     e = launch_dft(f, cx, DftMode{0, nullptr, nullptr}, st);
     if (e == cudaSuccess)
       e = launch_fast_fhat(cx.sb.ahat, cx.sb.bhat, x->C, x->n, x->npad, x->at<float>(x->off.fhat), st);
