@@ -241,6 +241,41 @@ __global__ void k_factors(const double* theta, int N, double dv, double* efac) {
   }
 }
 
+// Outputs of the transforms that a thread forms together: four share the loads of their common
+// operand and read the other one by one 16-byte load (the FP32 passes were bound by shared loads,
+// four for every 12 FP32 instructions; 128 cells, 32 velocities, five passes: 567 -> 396 us). FP64
+// is bound by its pipe and keeps single outputs. Every output is summed in the same order either
+// way, and the additions below name the product that is rounded, so that it doesn't depend on the
+// tile which one the compiler fuses: the increments of the defect-correction iteration amplify a
+// changed last bit to 3e-7.
+template <typename T>
+constexpr int kDftTile = sizeof(T) == 4 ? 4 : 1;
+template <typename T, int TR>
+__device__ __forceinline__ void load_tile_row(const T* p, T (&x)[TR]) {
+  if constexpr (TR == 4) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
+  } else {
+    x[0] = p[0];
+  }
+}
+__device__ __forceinline__ float mul_add(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mul_add(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_only(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_only(double a, double b) { return __dmul_rn(a, b); }
+// (re, im) += (x, y) (c - i s)
+template <typename T>
+__device__ __forceinline__ void dft_add(T& re, T& im, T x, T y, T c, T s) {
+  re += mul_add(x, c, mul_only(y, s));
+  im += mul_add(y, c, -mul_only(x, s));
+}
+// (re, im) += (x, y) (c + i s)
+template <typename T>
+__device__ __forceinline__ void idft_add(T& re, T& im, T x, T y, T c, T s) {
+  re += mul_add(x, c, -mul_only(y, s));
+  im += mul_add(x, s, mul_only(y, c));
+}
+
 // ---------------------------------------------------------------------------------------
 // Forward DFT, fhat_k = N^-3 sum_v f(v) exp(-i 2 pi k j / N), one index at a time.
 // Pass 1 (index 3) forms a = f - M and b = f + M in FP64 and transforms them in T.
@@ -252,9 +287,11 @@ __global__ void __launch_bounds__(256) k_dft_i3(const double* __restrict__ f, Ce
   extern __shared__ __align__(16) unsigned char smraw[];
   int n = N - 1;
   T* cs = (T*)smraw;             // [N][n] cos, transposed: k3 fastest, so that the threads of
-  T* sn = cs + n * N;            // [N][n] sin  a warp (consecutive k3) read consecutive banks
-  T* sa = sn + n * N;            // [N][N] a slab (i2, i3)
-  T* sbb = sa + N * N;           // [N][N] b slab
+  T* sn = cs + (n * N + 3) / 4 * 4;  // [N][n] sin  a warp (consecutive k3) read consecutive banks
+  constexpr int TR = kDftTile<T>;
+  const int NS = N + TR;         // row stride of the slabs: rows stay aligned, the stores spread over banks
+  T* sa = sn + (n * N + 3) / 4 * 4;  // [i3][i2] a slab
+  T* sbb = sa + N * NS;          // [i3][i2] b slab
   // M = E1[i1] E2[i2] E3[i3]: E12[i2] = E1[i1] E2[i2] for this block's i1, then one product
   __shared__ double E12[kMaxN], E3[kMaxN], E12r[kMaxN], E3r[kMaxN];
   int c = blockIdx.x, i1 = blockIdx.y;
@@ -282,17 +319,17 @@ __global__ void __launch_bounds__(256) k_dft_i3(const double* __restrict__ f, Ce
     double M = E12[i2] * E3[i3];
     double x = fc[t];
     if (md.mode == 0) {  // a = f - M, b = f + M
-      sa[t] = (T)(x - M);
-      sbb[t] = (T)(x + M);
+      sa[i3 * NS + i2] = (T)(x - M);
+      sbb[i3 * NS + i2] = (T)(x + M);
     } else {  // increments against the reference state f_ref, M_ref (exact in FP64, then rounded)
       double Mr = E12r[i2] * E3r[i3];
       double xr = md.f_ref[off + t];
       if (md.mode == 1) {  // a = (f - M) - (f_ref - M_ref), b = f + M
-        sa[t] = (T)((x - xr) - (M - Mr));
-        sbb[t] = (T)(x + M);
+        sa[i3 * NS + i2] = (T)((x - xr) - (M - Mr));
+        sbb[i3 * NS + i2] = (T)(x + M);
       } else {  // a unused, b = (f + M) - (f_ref + M_ref)
-        sa[t] = (T)0;
-        sbb[t] = (T)((x - xr) + (M - Mr));
+        sa[i3 * NS + i2] = (T)0;
+        sbb[i3 * NS + i2] = (T)((x - xr) + (M - Mr));
       }
     }
   }
@@ -300,19 +337,29 @@ __global__ void __launch_bounds__(256) k_dft_i3(const double* __restrict__ f, Ce
   typedef typename CplxOf<T>::type CT;
   CT* oa = sb.st1a + ((long long)c * N + i1) * N * n;
   CT* ob = sb.st1b + ((long long)c * N + i1) * N * n;
-  for (int t = threadIdx.x; t < N * n; t += blockDim.x) {
-    int i2 = t / n, k3 = t % n;
-    T ar = 0, ai = 0, br = 0, bi = 0;
+  for (int t = threadIdx.x; t < N / TR * n; t += blockDim.x) {
+    const int i2 = t / n * TR, k3 = t % n;
+    T ar[TR], ai[TR], br[TR], bi[TR];
+#pragma unroll
+    for (int q = 0; q < TR; q++) ar[q] = ai[q] = br[q] = bi[q] = 0;
     for (int i3 = 0; i3 < N; i3++) {
-      T co = cs[i3 * n + k3], si = sn[i3 * n + k3];
-      T a = sa[i2 * N + i3], b = sbb[i2 * N + i3];
-      ar += a * co;
-      ai -= a * si;
-      br += b * co;
-      bi -= b * si;
+      const T co = cs[i3 * n + k3], si = sn[i3 * n + k3];
+      T a[TR], b[TR];
+      load_tile_row<T, TR>(sa + i3 * NS + i2, a);
+      load_tile_row<T, TR>(sbb + i3 * NS + i2, b);
+#pragma unroll
+      for (int q = 0; q < TR; q++) {
+        ar[q] += a[q] * co;
+        ai[q] -= a[q] * si;
+        br[q] += b[q] * co;
+        bi[q] -= b[q] * si;
+      }
     }
-    oa[t] = make_cplx(ar, ai);
-    ob[t] = make_cplx(br, bi);
+#pragma unroll
+    for (int q = 0; q < TR; q++) {
+      oa[(i2 + q) * n + k3] = make_cplx(ar[q], ai[q]);
+      ob[(i2 + q) * n + k3] = make_cplx(br[q], bi[q]);
+    }
   }
 }
 
@@ -322,15 +369,18 @@ __global__ void __launch_bounds__(256) k_dft_i2(SpecBufs<T> sb, int N) {
   typedef typename CplxOf<T>::type CT;
   extern __shared__ __align__(16) unsigned char smraw[];
   int n = N - 1;
-  T* cs = (T*)smraw;
-  T* sn = cs + n * N;
-  CT* xa = (CT*)(sn + n * N);  // [N][n]
+  constexpr int TR = kDftTile<T>;
+  const int NS = (n + TR - 1) / TR * TR;  // outputs, padded to whole tiles
+  T* cs = (T*)smraw;    // [i][k] cos
+  T* sn = cs + NS * N;  // [i][k] sin
+  CT* xa = (CT*)(sn + NS * N);  // [N][n]
   CT* xb = xa + N * n;
   int c = blockIdx.x, i1 = blockIdx.y;
   if (!cell_active(sb.active, sb.cell_inst, c)) return;
-  for (int t = threadIdx.x; t < n * N; t += blockDim.x) {
-    cs[t] = sb.twc[t];
-    sn[t] = sb.tws[t];
+  for (int t = threadIdx.x; t < NS * N; t += blockDim.x) {
+    const int i = t / NS, k = t % NS;
+    cs[t] = k < n ? sb.twc[k * N + i] : (T)0;
+    sn[t] = k < n ? sb.tws[k * N + i] : (T)0;
   }
   const CT* ia = sb.st1a + ((long long)c * N + i1) * N * n;
   const CT* ib = sb.st1b + ((long long)c * N + i1) * N * n;
@@ -341,19 +391,28 @@ __global__ void __launch_bounds__(256) k_dft_i2(SpecBufs<T> sb, int N) {
   __syncthreads();
   CT* oa = sb.st2a + ((long long)c * N + i1) * n * n;
   CT* ob = sb.st2b + ((long long)c * N + i1) * n * n;
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    int k2 = t / n, k3 = t % n;
-    T ar = 0, ai = 0, br = 0, bi = 0;
+  for (int t = threadIdx.x; t < NS / TR * n; t += blockDim.x) {
+    const int k2 = t / n * TR, k3 = t % n;
+    T ar[TR], ai[TR], br[TR], bi[TR];
+#pragma unroll
+    for (int q = 0; q < TR; q++) ar[q] = ai[q] = br[q] = bi[q] = 0;
     for (int i2 = 0; i2 < N; i2++) {
-      T co = cs[k2 * N + i2], si = -sn[k2 * N + i2];
-      CT a = xa[i2 * n + k3], b = xb[i2 * n + k3];
-      ar += a.x * co - a.y * si;
-      ai += a.x * si + a.y * co;
-      br += b.x * co - b.y * si;
-      bi += b.x * si + b.y * co;
+      T co[TR], si[TR];
+      load_tile_row<T, TR>(cs + i2 * NS + k2, co);
+      load_tile_row<T, TR>(sn + i2 * NS + k2, si);
+      const CT a = xa[i2 * n + k3], b = xb[i2 * n + k3];
+#pragma unroll
+      for (int q = 0; q < TR; q++) {
+        dft_add(ar[q], ai[q], a.x, a.y, co[q], si[q]);
+        dft_add(br[q], bi[q], b.x, b.y, co[q], si[q]);
+      }
     }
-    oa[t] = make_cplx(ar, ai);
-    ob[t] = make_cplx(br, bi);
+#pragma unroll
+    for (int q = 0; q < TR; q++)
+      if (k2 + q < n) {
+        oa[(k2 + q) * n + k3] = make_cplx(ar[q], ai[q]);
+        ob[(k2 + q) * n + k3] = make_cplx(br[q], bi[q]);
+      }
   }
 }
 
@@ -363,15 +422,18 @@ __global__ void __launch_bounds__(256) k_dft_i1(SpecBufs<T> sb, int N) {
   typedef typename CplxOf<T>::type CT;
   extern __shared__ __align__(16) unsigned char smraw[];
   int n = N - 1;
-  T* cs = (T*)smraw;
-  T* sn = cs + n * N;
-  CT* xa = (CT*)(sn + n * N);  // [N][n] (i1, k3)
+  constexpr int TR = kDftTile<T>;
+  const int NS = (n + TR - 1) / TR * TR;  // outputs, padded to whole tiles
+  T* cs = (T*)smraw;    // [i][k] cos
+  T* sn = cs + NS * N;  // [i][k] sin
+  CT* xa = (CT*)(sn + NS * N);  // [N][n] (i1, k3)
   CT* xb = xa + N * n;
   int c = blockIdx.x, k2 = blockIdx.y;
   if (!cell_active(sb.active, sb.cell_inst, c)) return;
-  for (int t = threadIdx.x; t < n * N; t += blockDim.x) {
-    cs[t] = sb.twc[t];
-    sn[t] = sb.tws[t];
+  for (int t = threadIdx.x; t < NS * N; t += blockDim.x) {
+    const int i = t / NS, k = t % NS;
+    cs[t] = k < n ? sb.twc[k * N + i] : (T)0;
+    sn[t] = k < n ? sb.tws[k * N + i] : (T)0;
   }
   for (int t = threadIdx.x; t < N * n; t += blockDim.x) {
     int i1 = t / n, k3 = t % n;
@@ -383,20 +445,29 @@ __global__ void __launch_bounds__(256) k_dft_i1(SpecBufs<T> sb, int N) {
   T scale = (T)(1.0 / ((double)N * N * N));
   int g = c / kLanes, lane = c % kLanes;
   const int ls = g == sb.fold_group ? sb.fold_lanes : kLanes;  // lanes of the group's rows (SpecBufs)
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    int k1 = t / n, k3 = t % n;
-    T ar = 0, ai = 0, br = 0, bi = 0;
+  for (int t = threadIdx.x; t < NS / TR * n; t += blockDim.x) {
+    const int k1 = t / n * TR, k3 = t % n;
+    T ar[TR], ai[TR], br[TR], bi[TR];
+#pragma unroll
+    for (int q = 0; q < TR; q++) ar[q] = ai[q] = br[q] = bi[q] = 0;
     for (int i1 = 0; i1 < N; i1++) {
-      T co = cs[k1 * N + i1], si = -sn[k1 * N + i1];
-      CT a = xa[i1 * n + k3], b = xb[i1 * n + k3];
-      ar += a.x * co - a.y * si;
-      ai += a.x * si + a.y * co;
-      br += b.x * co - b.y * si;
-      bi += b.x * si + b.y * co;
+      T co[TR], si[TR];
+      load_tile_row<T, TR>(cs + i1 * NS + k1, co);
+      load_tile_row<T, TR>(sn + i1 * NS + k1, si);
+      const CT a = xa[i1 * n + k3], b = xb[i1 * n + k3];
+#pragma unroll
+      for (int q = 0; q < TR; q++) {
+        dft_add(ar[q], ai[q], a.x, a.y, co[q], si[q]);
+        dft_add(br[q], bi[q], b.x, b.y, co[q], si[q]);
+      }
     }
-    long long o = (long long)g * n * n * n * kLanes + (((long long)k1 * n + k2) * n + k3) * ls + lane;
-    sb.ahat[o] = make_cplx(ar * scale, ai * scale);
-    sb.bhat[o] = make_cplx(br * scale, bi * scale);
+#pragma unroll
+    for (int q = 0; q < TR; q++)
+      if (k1 + q < n) {
+        const long long o = (long long)g * n * n * n * kLanes + (((long long)(k1 + q) * n + k2) * n + k3) * ls + lane;
+        sb.ahat[o] = make_cplx(ar[q] * scale, ai[q] * scale);
+        sb.bhat[o] = make_cplx(br[q] * scale, bi[q] * scale);
+      }
   }
 }
 
@@ -863,16 +934,22 @@ __global__ void __launch_bounds__(256) k_idft_k1(SpecBufs<T> sb, int N) {
   }
   __syncthreads();
   CT* o = sb.st2a + (long long)c * N * n * n;  // [i1][k2][k3]
-  for (int t = threadIdx.x; t < N * n; t += blockDim.x) {
-    int i1 = t / n, k3 = t % n;
-    T re = 0, im = 0;
+  constexpr int TR = kDftTile<T>;
+  for (int t = threadIdx.x; t < N / TR * n; t += blockDim.x) {
+    const int i1 = t / n * TR, k3 = t % n;
+    T re[TR], im[TR];
+#pragma unroll
+    for (int q = 0; q < TR; q++) re[q] = im[q] = 0;
     for (int k1 = 0; k1 < n; k1++) {
-      T co = cs[k1 * N + i1], si = sn[k1 * N + i1];
-      CT q = x[k1 * n + k3];
-      re += q.x * co - q.y * si;
-      im += q.x * si + q.y * co;
+      T co[TR], si[TR];
+      load_tile_row<T, TR>(cs + k1 * N + i1, co);
+      load_tile_row<T, TR>(sn + k1 * N + i1, si);
+      const CT v = x[k1 * n + k3];
+#pragma unroll
+      for (int q = 0; q < TR; q++) idft_add(re[q], im[q], v.x, v.y, co[q], si[q]);
     }
-    o[((long long)i1 * n + k2) * n + k3] = make_cplx(re, im);
+#pragma unroll
+    for (int q = 0; q < TR; q++) o[((long long)(i1 + q) * n + k2) * n + k3] = make_cplx(re[q], im[q]);
   }
 }
 
@@ -894,16 +971,22 @@ __global__ void __launch_bounds__(256) k_idft_k2(SpecBufs<T> sb, int N) {
   for (int t = threadIdx.x; t < n * n; t += blockDim.x) x[t] = src[t];
   __syncthreads();
   CT* o = sb.st1a + ((long long)c * N + i1) * N * n;  // [i2][k3]
-  for (int t = threadIdx.x; t < N * n; t += blockDim.x) {
-    int i2 = t / n, k3 = t % n;
-    T re = 0, im = 0;
+  constexpr int TR = kDftTile<T>;
+  for (int t = threadIdx.x; t < N / TR * n; t += blockDim.x) {
+    const int i2 = t / n * TR, k3 = t % n;
+    T re[TR], im[TR];
+#pragma unroll
+    for (int q = 0; q < TR; q++) re[q] = im[q] = 0;
     for (int k2 = 0; k2 < n; k2++) {
-      T co = cs[k2 * N + i2], si = sn[k2 * N + i2];
-      CT q = x[k2 * n + k3];
-      re += q.x * co - q.y * si;
-      im += q.x * si + q.y * co;
+      T co[TR], si[TR];
+      load_tile_row<T, TR>(cs + k2 * N + i2, co);
+      load_tile_row<T, TR>(sn + k2 * N + i2, si);
+      const CT v = x[k2 * n + k3];
+#pragma unroll
+      for (int q = 0; q < TR; q++) idft_add(re[q], im[q], v.x, v.y, co[q], si[q]);
     }
-    o[t] = make_cplx(re, im);
+#pragma unroll
+    for (int q = 0; q < TR; q++) o[(i2 + q) * n + k3] = make_cplx(re[q], im[q]);
   }
 }
 
@@ -1160,8 +1243,8 @@ __global__ void k_build_weights(const int4* units, const long long* unit_step0, 
 template <typename T>
 static size_t dft_smem(int N, int extra_cplx, int extra_real) {
   typedef typename CplxOf<T>::type CT;
-  int n = N - 1;
-  return 2 * n * N * sizeof(T) + extra_cplx * sizeof(CT) + extra_real * sizeof(T);
+  // tables of at most N x N (padded tiles), then the slabs
+  return 2 * N * N * sizeof(T) + extra_cplx * sizeof(CT) + extra_real * sizeof(T);
 }
 
 template <typename T, int BK, int F>
@@ -1256,7 +1339,7 @@ cudaError_t launch_dft(const double* f, const CollideCtx<T>& x, const DftMode& m
   // the factors of this step were written by launch_moments, those of the reference by the first
   // of the two transforms of an increment
   if (md.mode == 1) k_factors<<<C, 3 * N, 0, st>>>(md.theta_ref, N, x.dv, x.efac_ref);
-  size_t sm1 = dft_smem<T>(N, 0, 2 * N * N);
+  size_t sm1 = dft_smem<T>(N, 0, 2 * N * (N + kDftTile<T>));
   e = func_attr((const void*)k_dft_i3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
   if (e != cudaSuccess) return e;
   k_dft_i3<T><<<dim3(C, N), 256, sm1, st>>>(f, x.ct, x.efac, x.efac_ref, x.sb, N, x.dv, md);
