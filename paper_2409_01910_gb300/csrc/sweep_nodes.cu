@@ -6,7 +6,16 @@
 // to 4e-14, the Q of two defect-correction iterations differs by 3e-7 from the one with this
 // kernel (the error of either against 64 bits is 8.5e-7). The iterates of sgs_dc_step, whose
 // results callers compare between versions, therefore keep their scan; every other call runs
-// k_sweep, which takes a quarter of the time (64 cells of 32^3: 2.5 instead of 10.9 ms).
+// k_sweep, which is faster still (from a cold start, 64 cells of 32^3: 2.4 instead of 10.7 ms with
+// this kernel's first form).
+//
+// A visit is a serial chain: Newton evaluations (some 40) and cluster reductions (2 us each). It is
+// bound by the latency of that chain, and an FP64 instruction, which holds its scheduler for 64
+// cycles (a conversion: 101), is its dearest link. So a decision is taken in FP32 where that leaves
+// no doubt, widening to FP64 is done by integer operations, components are spread over lanes, and a
+// warp sum takes 9 double-float additions (warp_sums) instead of 25 to 35. All of it keeps the bits.
+// A visit of the defect correction (64 cells, 32 velocities): 85 -> 55 us, two iterations of
+// sgs_dc_step 89.4 -> 74.0 ms.
 //
 // One thread-block cluster walks the instance's cells in scan order inside a single launch.
 // Each thread owns EPT consecutive velocity nodes of one pencil (fixed i1, i2) in every cell.
@@ -31,7 +40,6 @@ struct NodesSmem {
   E vv[kMaxN];         // nodes v_i
   E vq[kMaxN];         // v_i^2
   E c1e[kMaxN];        // |v_i| / dx (step-1 weights, x part)
-  E c2e[kMaxN];        // |v_i| / dy (step-1 weights, y part; 2-D)
   E den[kMaxN];        // 1 / (|v_i|/dx + nu/eps) of the current cell
   E c1A[kMaxN];        // |v_i|/dx + nu/eps of the current cell
   E ef[3][kMaxN];      // factors of the last Newton evaluation (ef[0] carries exp(alpha))
@@ -39,8 +47,7 @@ struct NodesSmem {
   E Ep[3][kMaxN];      // factors of the step-1 Maxwellian
   E S[3][5];           // 1-D sums of the last evaluation (unweighted)
   E S1w[5];            // dimension-1 sums with the step-1 weights |v1|/dx, same evaluation
-  E S2w[5];            // dimension-2 sums with the weights |v2|/dy (2-D), same evaluation
-  E Sb[2][5][5];       // Newton evaluations, double-buffered: row r = sums of evaluating warp r
+  E Sb[2][4][5];       // Newton evaluations, double-buffered: row r = sums of evaluating warp r
   E Gs[3][6];          // per-dimension sums for the norm of M+ - M[g] (derived residual)
   E svE[5];            // step-1 target s
   E W3[4][kMaxN];      // third factor of each wall's unit Maxwellian
@@ -50,14 +57,62 @@ struct NodesSmem {
   E scal[6];           // per-visit scalars: wall densities of the sides, nu/eps
   double red_part[2][kRedMax];
   double red_tot[kRedMax];
-  double thg[5], thp[5], th_try[5], dir[5];
-  float fn;
-  float stepf;         // exponent change of the full Newton step
-  int flag;
+  double thg[5], thp[5];
   int ctl;             // broadcast decisions of thread 0
-  int wdims;           // space dimensions of the step-1 weights (1: |v1|/dx; 2: + |v2|/dy)
   int nret;            // Newton result, for the warps that do not evaluate
 };
+
+// The double of an FP32 number, and of a double-float, with the bits of the conversion: a normal
+// number is widened by integer operations (a conversion holds the FP64 unit for 101 cycles).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)x;  // subnormal, infinite, NaN
+  const unsigned hi = (u & 0x80000000u) | (m == 0u ? 0u : (m >> 3) + 0x38000000u);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(dfloat x) { return widen(x.hi) + widen(x.lo); }
+
+__device__ __forceinline__ float shfl_i(float v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+__device__ __forceinline__ dfloat shfl_i(dfloat v, int lane) { return {shfl_i(v.hi, lane), shfl_i(v.lo, lane)}; }
+
+// Sums over the warp of NV <= 8 values per lane: lane l returns the total of value l / 4. The
+// additions are those of a butterfly over all values (warp_allsum: the same pairs at every level,
+// and an addition is commutative), but in each of the first three steps a lane keeps half of its
+// values and hands over the other half, so there are 9 of them instead of 5 NV.
+template <int NV, typename E>
+__device__ __forceinline__ E warp_sums(const E (&x)[NV], int lane) {
+  E v[8];
+#pragma unroll
+  for (int q = 0; q < 8; q++) v[q] = q < NV ? x[q] : cvt<E>(0.0);
+  int o = 16;
+#pragma unroll
+  for (int h = 4; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int q = 0; q < h; q++) {
+      const E send = up ? v[q] : v[q + h];
+      const E keep = up ? v[q + h] : v[q];
+      v[q] = keep + shfl_x(send, o);
+    }
+  }
+  v[0] += shfl_x(v[0], 2);
+  v[0] += shfl_x(v[0], 1);
+  return v[0];
+}
+
+// Whether x < lim where FP32 leaves no doubt (x off by at most 1e-5 mag): 1 yes, 0 no, -1 open
+// (also for NaN, infinities and the ends of the range).
+__device__ __forceinline__ int clearly_less(float x, float mag, float lim) {
+  if (!(lim > 1e-25f && lim < 1e25f)) return -1;
+  if (!(fabsf(x - lim) > 1e-5f * (mag + lim))) return -1;
+  return x < lim ? 1 : 0;
+}
+// Existence test of step 1 (eq. (26)), f0 > 0 and f0 f4 > f1^2 + f2^2 + f3^2, the same way.
+__device__ __forceinline__ int clearly_exists(float f0, float f1, float f2, float f3, float f4) {
+  const float pl = f0 * f4, mi = f1 * f1 + f2 * f2 + f3 * f3, mag = fabsf(pl) + mi;
+  if (!(mag > 1e-25f && mag < 1e25f && fabsf(pl - mi) > 1e-5f * mag)) return -1;
+  return f0 > 0.0f && pl > mi ? 1 : 0;
+}
 
 // ---------------------------------------------------------------------------------------
 // Cluster-wide sum of NV values per thread; tot (double) and sm.red_tote (E) receive the
@@ -66,17 +121,14 @@ struct NodesSmem {
 template <int NV, typename E>
 __device__ inline void cluster_reduce(E (&v)[NV], double (&tot)[NV], NodesSmem<E>& sm, int& buf,
                                       cg::cluster_group& cl, int CS) {
-  warp_allsum<NV, E>(v);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (lane == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; q++) sm.red_warp[wid][q] = v[q];
-  }
+  const E ws = warp_sums<NV, E>(v, lane);
+  if ((lane & 3) == 0 && (lane >> 2) < NV) sm.red_warp[wid][lane >> 2] = ws;
   __syncthreads();
   if (threadIdx.x < NV) {
     E t = sm.red_warp[0][threadIdx.x];
     for (int k = 1; k < nw; k++) t += sm.red_warp[k][threadIdx.x];
-    sm.red_part[buf][threadIdx.x] = tod(t);
+    sm.red_part[buf][threadIdx.x] = widen(t);
   }
   cl.sync();
   // one thread per (value q, rank r): lanes of a warp hold segments of CS consecutive ranks
@@ -108,10 +160,9 @@ __device__ inline void cluster_reduce(E (&v)[NV], double (&tot)[NV], NodesSmem<E
 template <typename E>
 __device__ __noinline__ void eval_cta(NodesSmem<E>& sm, int N) {
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (wid < 3 + sm.wdims) {
-    // warps 0-2: dimension d; warp 3: dimension 1 again, weighted by |v1|/dx; warp 4 (2-D):
-    // dimension 2 again, weighted by |v2|/dy (step 1, eq. (24))
-    const int d = wid == 3 ? 0 : (wid == 4 ? 1 : wid);
+  if (wid < 4) {
+    // warps 0-2: dimension d; warp 3: dimension 1 again, weighted by |v1|/dx (step 1, eq. (24))
+    const int d = wid == 3 ? 0 : wid;
     E e = cvt<E>(0.0);
     if (lane < N) {
       E x = sm.thE[1 + d] * sm.vv[lane] - sm.thE[4] * sm.vq[lane];
@@ -120,26 +171,14 @@ __device__ __noinline__ void eval_cta(NodesSmem<E>& sm, int N) {
     }
     if (wid < 3) sm.ef[d][lane] = e;
     if (wid == 3) e = e * sm.c1e[lane];
-    if (wid == 4) e = e * sm.c2e[lane];
     E s[5];
     s[0] = e;
     s[1] = e * sm.vv[lane];
     s[2] = e * sm.vq[lane];
     s[3] = s[2] * sm.vv[lane];
     s[4] = s[2] * sm.vq[lane];
-    warp_allsum<5, E>(s);
-    if (lane < 5) {
-      E t = s[0];
-#pragma unroll
-      for (int q = 1; q < 5; q++)
-        if (lane == q) t = s[q];
-      if (wid < 3)
-        sm.S[d][lane] = t;
-      else if (wid == 3)
-        sm.S1w[lane] = t;
-      else
-        sm.S2w[lane] = t;
-    }
+    const E t = warp_sums<5, E>(s, lane);
+    if ((lane & 3) == 0 && lane < 20) (wid < 3 ? sm.S[d] : sm.S1w)[lane >> 2] = t;
   }
   __syncthreads();
 }
@@ -173,18 +212,6 @@ __device__ inline void moments_from_sums(const E* S1, const E* S2, const E* S3, 
   for (int i = 0; i < 15; i++) Aa[i] = t[i];
 }
 
-// Moment k of the separable Maxwellian from its three 1-D sums, the same expression as
-// moments_from_sums gives for component k.
-template <typename E>
-__device__ inline E moment_k(const E* S1, const E* S2, const E* S3, int k) {
-  const E s23 = S2[0] * S3[0];
-  if (k == 0) return S1[0] * s23;
-  if (k == 1) return S1[1] * s23;
-  if (k == 2) return S1[0] * (S2[1] * S3[0]);
-  if (k == 3) return S1[0] * (S2[0] * S3[1]);
-  return S1[2] * s23 + S1[0] * (S2[2] * S3[0] + S2[0] * S3[2]);
-}
-
 // Component k of a five-element register array (static indices only).
 template <typename E>
 __device__ inline E pick5(const E (&v)[5], int k) {
@@ -195,95 +222,67 @@ __device__ inline E pick5(const E (&v)[5], int k) {
   return r;
 }
 
-// Warp 0: residual F (E), Jacobian (FP32) and the scaled residual norm from the 1-D sums.
-// wmode 0: plain weights w; 1: w |v1|/dx; 2: w (|v1|/dx + |v2|/dy), a sum of two separable
-// terms.
+// Lane k < 5 returns moment k, with the operations of moments_from_sums (lanes 5 and 6 form parts of
+// the last one), so that a warp does a handful of double-float operations instead of forty.
 template <typename E>
-__device__ inline void combine(const NodesSmem<E>& sm, E w, int wmode, const E* target, E (&F)[5], float (&A)[15],
-                               float& fn) {
-  E mom[5];
-  float Aa[15];
-  moments_from_sums<E>(wmode ? sm.S1w : sm.S[0], sm.S[1], sm.S[2], mom, Aa);
-  if (wmode == 2) {
-    E m2[5];
-    float A2[15];
-    moments_from_sums<E>(sm.S[0], sm.S2w, sm.S[2], m2, A2);
-#pragma unroll
-    for (int i = 0; i < 5; i++) mom[i] += m2[i];
-#pragma unroll
-    for (int i = 0; i < 15; i++) Aa[i] += A2[i];
-  }
+__device__ __forceinline__ E lane_moment(const E* S1, const E* S2, const E* S3, int lane) {
+  const int i = lane == 1 ? 1 : (lane == 4 ? 2 : 0), j = lane == 2 ? 1 : (lane == 5 ? 2 : 0),
+            l = lane == 3 ? 1 : (lane == 6 ? 2 : 0);
+  E u = S2[j] * S3[l];
+  const E u6 = shfl_i(u, 6);
+  if (lane == 5) u = u + u6;
+  E x = S1[i] * u;
+  const E x5 = shfl_i(x, 5);
+  if (lane == 4) x = x + x5;
+  return x;
+}
+
+// Residual of the moments against the target (lane k: component k of it, tl), in Ff on every
+// lane, the Jacobian (FP32) and the scaled residual norm, from the 1-D sums. it0: |target_0|.
+template <typename E>
+__device__ __forceinline__ void combine(const E* S1, const E* S2, const E* S3, E w, E tl, float it0, float (&Ff)[5],
+                                        float (&A)[15], float& fn) {
+  const float Fl = tof(w * lane_moment<E>(S1, S2, S3, threadIdx.x & 31) - tl);
   float amax = 0.0f;
 #pragma unroll
   for (int i = 0; i < 5; i++) {
-    F[i] = w * mom[i] - target[i];
-    amax = fmaxf(amax, fabsf(tof(F[i])));
+    Ff[i] = shfl_i(Fl, i);
+    amax = fmaxf(amax, fabsf(Ff[i]));
   }
-  fn = amax / fabsf(tof(target[0]));
-  float cf = tof(w);
+  fn = amax / it0;
+  E mom[5];
+  float Aa[15];
+  moments_from_sums<E>(S1, S2, S3, mom, Aa);
+  const float cf = tof(w);
 #pragma unroll
   for (int i = 0; i < 15; i++) A[i] = cf * Aa[i];
 }
 
 // One evaluation by evaluating warp wid (warps 0-2: dimension wid, unweighted; warp 3:
-// dimension 1 weighted by |v1|/dx; warp 4: dimension 2 weighted by |v2|/dy) at the trial
-// theta thE: factors of warps 0-2 to sm.ef, the five 1-D sums to row wid of sm.Sb[buf].
-// The same arithmetic as eval_cta.
+// dimension 1 weighted by |v1|/dx) at the trial theta, of which lane k holds component k: factors
+// of warps 0-2 to sm.ef, the five 1-D sums to row wid of sm.Sb[buf]. The same arithmetic as
+// eval_cta.
 template <typename E>
-__device__ inline void eval_warp(NodesSmem<E>& sm, int N, const E (&thE)[5], int wid, int buf) {
+__device__ __forceinline__ void eval_warp(NodesSmem<E>& sm, int N, E thl, int wid, int buf) {
   const int lane = threadIdx.x & 31;
-  const int d = wid == 3 ? 0 : (wid == 4 ? 1 : wid);
+  const int d = wid == 3 ? 0 : wid;
+  const E b = shfl_i(thl, 1 + d), g = shfl_i(thl, 4), al = shfl_i(thl, 0);
   E e = cvt<E>(0.0);
   if (lane < N) {
-    E x = thE[1 + d] * sm.vv[lane] - thE[4] * sm.vq[lane];
-    if (d == 0) x += thE[0];
+    E x = b * sm.vv[lane] - g * sm.vq[lane];
+    if (d == 0) x += al;
     e = exp_in(x);
   }
   if (wid < 3) sm.ef[d][lane] = e;
   if (wid == 3) e = e * sm.c1e[lane];
-  if (wid == 4) e = e * sm.c2e[lane];
   E s[5];
   s[0] = e;
   s[1] = e * sm.vv[lane];
   s[2] = e * sm.vq[lane];
   s[3] = s[2] * sm.vv[lane];
   s[4] = s[2] * sm.vq[lane];
-  warp_allsum<5, E>(s);
-  if (lane < 5) {
-    E t = s[0];
-#pragma unroll
-    for (int q = 1; q < 5; q++)
-      if (lane == q) t = s[q];
-    sm.Sb[buf][wid][lane] = t;
-  }
-}
-
-// combine on the sums of one buffer (rows as in eval_warp).
-template <typename E>
-__device__ inline void combine_rows(const E (*R)[5], E w, int wmode, const E* target, E (&F)[5], float (&A)[15],
-                                    float& fn) {
-  E mom[5];
-  float Aa[15];
-  moments_from_sums<E>(wmode ? R[3] : R[0], R[1], R[2], mom, Aa);
-  if (wmode == 2) {
-    E m2[5];
-    float A2[15];
-    moments_from_sums<E>(R[0], R[4], R[2], m2, A2);
-#pragma unroll
-    for (int i = 0; i < 5; i++) mom[i] += m2[i];
-#pragma unroll
-    for (int i = 0; i < 15; i++) Aa[i] += A2[i];
-  }
-  float amax = 0.0f;
-#pragma unroll
-  for (int i = 0; i < 5; i++) {
-    F[i] = w * mom[i] - target[i];
-    amax = fmaxf(amax, fabsf(tof(F[i])));
-  }
-  fn = amax / fabsf(tof(target[0]));
-  float cf = tof(w);
-#pragma unroll
-  for (int i = 0; i < 15; i++) A[i] = cf * Aa[i];
+  const E t = warp_sums<5, E>(s, lane);
+  if ((lane & 3) == 0 && lane < 20) sm.Sb[buf][wid][lane >> 2] = t;
 }
 
 // Barrier among the evaluating warps only (hardware barrier 1; __syncthreads uses 0).
@@ -292,43 +291,42 @@ __device__ __forceinline__ void eval_bar(int nwarps) {
 }
 
 // Newton from the theta in th (shared memory). With have_eval the last evaluation (sm.S,
-// sm.S1w, sm.S2w, sm.ef) is already at th and is reused. On success th holds the root, the
+// sm.S1w, sm.ef) is already at th and is reused. On success th holds the root, the
 // last evaluation is at th, and the return value is the iteration count; -1 on failure.
+// weighted: the step-1 weights |v1|/dx.
 //
-// Only the evaluating warps (3 + wdims) take part, and each of them runs the whole iteration
+// Only the four evaluating warps take part, and each of them runs the whole iteration
 // itself: it evaluates its dimension into a double-buffered row of sm.Sb, meets the others
 // at one barrier, and then combines the rows, factorises the Jacobian (FP32: inexact Newton)
 // and takes the line-search decisions in registers. All of them read the same rows and the
 // same inputs through the same instructions, so their decisions agree and they pass every
 // barrier the same number of times; one barrier per evaluation replaces the CTA barriers
-// and thread-0 broadcasts of a split design. The FP64 trial theta is formed on lane 0 of
-// each warp and shuffled to its lanes (FP64 is scarce on this GPU).
+// and thread-0 broadcasts of a split design. The FP64 theta is spread over the lanes (lane k:
+// component k), the moments and sums too, so an iteration takes one FP64 instruction. With every
+// component on lane 0 it took five of them and six conversions, about half of its 1.5 us.
 template <typename E>
-__device__ __noinline__ int newton_cta(NodesSmem<E>& sm, int N, E w, int wmode, const E* target, double* th,
+__device__ __noinline__ int newton_cta(NodesSmem<E>& sm, int N, E w, bool weighted, const E* target, double* th,
                                        double L, double tol, int maxit, bool have_eval) {
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nev = 3 + sm.wdims;
+  constexpr int nev = 4;
   // Converged as well once the scaled moment residual |F|/rho is at the arithmetic's
-  // resolution (double-float and FP64 evaluate F to about 1e-14; 1e-13 bounds the relative
+  // resolution (double-float evaluates F to about 1e-14; 1e-13 bounds the relative
   // error of the Maxwellian near 1e-12 or below): with the residual already
   // there, a further step could only confirm it.
-  constexpr float ftol = sizeof(E) == 4 ? 0.0f : 1e-13f;
+  constexpr float ftol = 1e-13f;
   if (wid < nev) {
-    double thc[5];
-#pragma unroll
-    for (int k = 0; k < 5; k++) thc[k] = th[k];
-    E F[5];
-    float A[15], fn = 0.0f;
+    const int kl = min(lane, 4);  // this lane's component
+    double thl = th[kl];
+    const E tl = pick5<E>(*reinterpret_cast<const E(*)[5]>(target), kl);
+    const float it0 = fabsf(tof(target[0]));
+    float Ff[5], A[15], fn = 0.0f;
     int buf = 0, last = -1;  // last: buffer of the latest evaluation (-1: the canonical sums)
     if (have_eval) {
-      combine<E>(sm, w, wmode, target, F, A, fn);
+      combine<E>(weighted ? sm.S1w : sm.S[0], sm.S[1], sm.S[2], w, tl, it0, Ff, A, fn);
     } else {
-      E thE[5];
-#pragma unroll
-      for (int k = 0; k < 5; k++) thE[k] = cvt<E>(thc[k]);
-      eval_warp<E>(sm, N, thE, wid, buf);
+      eval_warp<E>(sm, N, cvt<E>(thl), wid, buf);
       eval_bar(nev);
-      combine_rows<E>(sm.Sb[buf], w, wmode, target, F, A, fn);
+      combine<E>(sm.Sb[buf][weighted ? 3 : 0], sm.Sb[buf][1], sm.Sb[buf][2], w, tl, it0, Ff, A, fn);
       last = buf;
       buf ^= 1;
     }
@@ -337,30 +335,21 @@ __device__ __noinline__ int newton_cta(NodesSmem<E>& sm, int N, E w, int wmode, 
       ret = -1;
       float fn_cur = fn;
       for (int it = 0; it < maxit; it++) {
-        float y[5], Ff[5];
-#pragma unroll
-        for (int i = 0; i < 5; i++) Ff[i] = tof(F[i]);
+        float y[5];
         if (!chol5_solve(A, Ff, y)) break;
         // exponent change of a full step, |d alpha| + L sum |d beta| + L^2 |d gamma|
         const float Lf = (float)L;
         const float stepf = fabsf(y[0]) + Lf * (fabsf(y[1]) + fabsf(y[2]) + fabsf(y[3])) + Lf * Lf * fabsf(y[4]);
         // -D A^{-1} F, D = diag(1,1,1,1,-1)
-        const double dir[5] = {-(double)y[0], -(double)y[1], -(double)y[2], -(double)y[3], (double)y[4]};
+        const float yl = pick5<float>(y, kl);
+        const double dirl = widen(kl == 4 ? yl : -yl);
         float lam = 1.0f;
-        double tt[5];
+        double lamd = 1.0, tt;
         for (int hv = 0; hv < 40; hv++) {
-          E thE[5];
-#pragma unroll
-          for (int k = 0; k < 5; k++) {
-            double t = 0.0;
-            if (lane == 0) t = thc[k] + (double)lam * dir[k];
-            t = __shfl_sync(0xffffffffu, t, 0);
-            tt[k] = t;
-            thE[k] = cvt<E>(t);
-          }
-          eval_warp<E>(sm, N, thE, wid, buf);
+          tt = fma(lamd, dirl, thl);
+          eval_warp<E>(sm, N, cvt<E>(tt), wid, buf);
           eval_bar(nev);
-          combine_rows<E>(sm.Sb[buf], w, wmode, target, F, A, fn);
+          combine<E>(sm.Sb[buf][weighted ? 3 : 0], sm.Sb[buf][1], sm.Sb[buf][2], w, tl, it0, Ff, A, fn);
           last = buf;
           buf ^= 1;
           if (fn == fn && (fn <= fn_cur || fn <= 1e-10f)) {
@@ -368,10 +357,10 @@ __device__ __noinline__ int newton_cta(NodesSmem<E>& sm, int N, E w, int wmode, 
             break;
           }
           lam *= 0.5f;
+          lamd *= 0.5;
         }
         const float step = lam * stepf;
-#pragma unroll
-        for (int k = 0; k < 5; k++) thc[k] = tt[k];
+        thl = tt;
         if (!(step == step)) break;
         if (step <= (float)tol || fn_cur <= ftol) {
           ret = it + 1;
@@ -382,18 +371,10 @@ __device__ __noinline__ int newton_cta(NodesSmem<E>& sm, int N, E w, int wmode, 
     // publish the result: theta, and the latest evaluation's sums as the canonical ones (its
     // factors are in sm.ef already)
     if (wid == 0 && lane < 5) {
-      th[lane] = thc[lane];
-      sm.thE[lane] = cvt<E>(thc[lane]);
+      th[lane] = thl;
+      sm.thE[lane] = cvt<E>(thl);
     }
-    if (last >= 0 && lane < 5) {
-      const E t = sm.Sb[last][wid][lane];
-      if (wid < 3)
-        sm.S[wid][lane] = t;
-      else if (wid == 3)
-        sm.S1w[lane] = t;
-      else
-        sm.S2w[lane] = t;
-    }
+    if (last >= 0 && lane < 5) (wid < 3 ? sm.S[wid] : sm.S1w)[lane] = sm.Sb[last][wid][lane];
     if (wid == 0 && lane == 0) sm.nret = ret;
   }
   __syncthreads();
@@ -426,7 +407,7 @@ __device__ __noinline__ int solve_mg(NodesSmem<E>& sm, int N, E w, const E* mom,
   if (th0) {
     if (tid < 5) sm.thg[tid] = keep[tid];
     __syncthreads();
-    it = newton_cta<E>(sm, N, w, 0, mom, sm.thg, L, tol, maxit, have_eval);
+    it = newton_cta<E>(sm, N, w, false, mom, sm.thg, L, tol, maxit, have_eval);
   }
   if (it < 0) {
     if (tid == 0) {
@@ -438,7 +419,7 @@ __device__ __noinline__ int solve_mg(NodesSmem<E>& sm, int N, E w, const E* mom,
     }
     __syncthreads();
     if (sm.ctl) {
-      it = newton_cta<E>(sm, N, w, 0, mom, sm.thg, L, tol, maxit, false);
+      it = newton_cta<E>(sm, N, w, false, mom, sm.thg, L, tol, maxit, false);
     } else {
       status |= SGS_ST_NONPOSITIVE;
     }
@@ -466,19 +447,13 @@ __device__ __noinline__ int solve_mg(NodesSmem<E>& sm, int N, E w, const E* mom,
 // M[g]'s). 1 + tau = 2, 4, 8, ...: the first target that passes eq. (26) replaces sd and
 // sm.svE. Returns whether one was found.
 template <typename E>
-__device__ inline bool relax_target(NodesSmem<E>& sm, E w, bool two_d, double (&sd)[5]) {
+__device__ inline bool relax_target(NodesSmem<E>& sm, E w, double (&sd)[5]) {
   E m1[5];
   float Aa[15];
   moments_from_sums<E>(sm.S1w, sm.S[1], sm.S[2], m1, Aa);
   double mw[5];
 #pragma unroll
   for (int k = 0; k < 5; k++) mw[k] = tod(w * m1[k]);
-  if (two_d) {
-    E m2[5];
-    moments_from_sums<E>(sm.S[0], sm.S2w, sm.S[2], m2, Aa);
-#pragma unroll
-    for (int k = 0; k < 5; k++) mw[k] += tod(w * m2[k]);
-  }
   for (double q = 2.0; q <= 1048576.0; q *= 2.0) {
     double t[5];
 #pragma unroll
@@ -512,14 +487,8 @@ __device__ inline void derived_sums(NodesSmem<E>& sm) {
   if (wid < 3) {
     const E p = sm.Ep[wid][lane], q = sm.Eg[wid][lane], dl = q - p;
     E x[6] = {p * p, p * dl, dl * dl, p * q, dl * q, q * q};
-    warp_allsum<6, E>(x);
-    if (lane < 6) {
-      E t = x[0];
-#pragma unroll
-      for (int k = 1; k < 6; k++)
-        if (lane == k) t = x[k];
-      sm.Gs[wid][lane] = t;
-    }
+    const E t = warp_sums<6, E>(x, lane);
+    if ((lane & 3) == 0 && lane < 24) sm.Gs[wid][lane >> 2] = t;
   }
   __syncthreads();
 }
@@ -532,6 +501,18 @@ __device__ inline E derived_norm2(const NodesSmem<E>& sm) {
   const E* c = sm.Gs[2];
   E cross = a[4] * b[1] * c[0] + a[4] * b[3] * c[1] + a[5] * b[4] * c[1];
   return a[2] * b[0] * c[0] + a[5] * b[2] * c[0] + a[5] * b[5] * c[2] + cvt<E>(2.0) * cross;
+}
+
+// The same in FP32, mag the sum of its terms' magnitudes (clearly_less).
+template <typename E>
+__device__ __forceinline__ float derived_norm2_f32(const NodesSmem<E>& sm, float& mag) {
+  float a[6], b[6], c[6];
+#pragma unroll
+  for (int k = 0; k < 6; k++) a[k] = tof(sm.Gs[0][k]), b[k] = tof(sm.Gs[1][k]), c[k] = tof(sm.Gs[2][k]);
+  const float x0 = a[4] * b[1] * c[0], x1 = a[4] * b[3] * c[1], x2 = a[5] * b[4] * c[1];
+  const float p = a[2] * b[0] * c[0] + a[5] * b[2] * c[0] + a[5] * b[5] * c[2];
+  mag = p + 2.0f * (fabsf(x0) + fabsf(x1) + fabsf(x2));
+  return p + 2.0f * (x0 + x1 + x2);
 }
 
 template <typename E, int EPT>
@@ -552,8 +533,9 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
   const int tid = threadIdx.x;
   const bool pfp = I.inner_method == SGS_PFP || I.inner_method == SGS_PFP_RELAX;
   const bool relax = I.inner_method == SGS_PFP_RELAX;
-  const bool lowp = sizeof(E) == 4;  // plain FP32: tolerances at FP32 resolution
-  const double ntol = lowp ? fmax(I.newton_tol, 1e-5) : I.newton_tol;
+  const double ntol = I.newton_tol;
+  // inner_tol^2 / w; a tolerance that is not positive leaves every decision to FP64
+  const float tol2f = I.inner_tol > 0.0 ? (float)I.tol2_w : -1.0f;
   const E inv_eps = cvt<E>(1.0 / I.eps);
   const E zero = cvt<E>(0.0);
   if (tid < kMaxN) {
@@ -561,11 +543,9 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
     sm.vv[tid] = cvt<E>(v);
     sm.vq[tid] = cvt<E>(v * v);
     sm.c1e[tid] = cvt<E>(fabs(v) * inv_dx);
-    sm.c2e[tid] = zero;
     sm.W3[0][tid] = cvt<E>(tid < N ? I.wall[0][2][tid] : 0.0);
     sm.W3[1][tid] = cvt<E>(tid < N ? I.wall[1][2][tid] : 0.0);
   }
-  if (tid == 0) sm.wdims = 1;
   __syncthreads();
 
   // this thread's nodes: pencil (i1, i2), i3 in [i30, i30 + EPT)
@@ -640,12 +620,13 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
     E mom[5];
 #pragma unroll
     for (int k = 0; k < 5; k++) mom[k] = w * sm.red_tote[k];
-    if (tid == 0) {
+    if (tid == 0 && lw)
       sm.scal[0] = cvt<E>(I.bc_kind[0] == SGS_INFLOW ? I.bc_rho[0] : -(wd * t7[5]) / I.wall_denom[0]);
+    if (tid == 0 && rw)
       sm.scal[1] = cvt<E>(I.bc_kind[1] == SGS_INFLOW ? I.bc_rho[1] : -(wd * t7[6]) / I.wall_denom[1]);
-    }
     __syncthreads();
-    const E rho_l = sm.scal[0], rho_r = sm.scal[1], Acoef = sm.scal[2];
+    const E rho_l = lw ? sm.scal[0] : zero, rho_r = rw ? sm.scal[1] : zero, Acoef = sm.scal[2];
+    const float limf = tol2f / (tof(Acoef) * tof(Acoef));  // bound of sum (M+ - M[g])^2
     const E c1A = sm.c1A[i1], den = sm.den[i1];
     if (own && wall_cell) form_r(rho_l, rho_r);
 
@@ -668,11 +649,26 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
     E momg[5];  // moments of the current iterate g
 #pragma unroll
     for (int k = 0; k < 5; k++) momg[k] = mom[k];
+    // whether the inner iteration stops: small 1 / 0, or 2 for a NaN residual (thread 0)
+    auto decide = [&](int small) {
+      bool stop;
+      if (I.inner_fixed > 0) {
+        stop = it >= I.inner_fixed;
+      } else {
+        stop = small == 1 || it >= I.inner_max;
+        if (stop && small != 1) status |= SGS_ST_INNER_CAP;
+      }
+      if (small == 2) {
+        status |= SGS_ST_NONFINITE;
+        stop = true;
+      }
+      return stop;
+    };
     for (;;) {
       if (!derived) {
-        // ---- pass B: cell-equation residual, its scale, and the step-1 target s (eq. (26))
+        // ---- pass B: cell-equation residual and the step-1 target s (eq. (26))
         E e12 = sm.Eg[0][i1] * sm.Eg[1][i2];
-        E rs = zero, sc = zero, b0 = zero, b3 = zero, b4 = zero;
+        E rs = zero, b0 = zero, b3 = zero, b4 = zero;
         if (own) {
 #pragma unroll
           for (int t = 0; t < EPT; t++) {
@@ -680,39 +676,37 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
             // (|v1|/dx) g + r - (nu/eps)(M - g) = (|v1|/dx + nu/eps) g + r - (nu/eps) M
             E res = c1A * g[t] + r[t] - Acoef * M;
             rs += res * res;
-            E mag = c1A * g[t];
-            sc += mag * mag;
             E tt = c1 * (M - g[t]) - r[t];
             b0 += tt;
             b3 += tt * sm.vv[i30 + t];
             b4 += tt * sm.vq[i30 + t];
           }
         }
-        E v7[7] = {rs, b0, v1 * b0, v2 * b0, b3, vq12 * b0 + b4, sc};
-        double t6[7];
-        cluster_reduce<7, E>(v7, t6, sm, buf, cl, CS);
+        E v6[6] = {rs, b0, v1 * b0, v2 * b0, b3, vq12 * b0 + b4};
+        double t6[6];
+        cluster_reduce<6, E>(v6, t6, sm, buf, cl, CS);
         // thread 0 decides: stop, and whether step 1 is attempted (existence test, eq. (26))
         if (tid == 0) {
-          const double res = sqrt(wd * t6[0]);
-          double tol = I.inner_tol;
-          if (lowp) tol = fmax(tol, 2e-6 * sqrt(wd * t6[6]));
-          bool stop;
-          if (I.inner_fixed > 0) {
-            stop = it >= I.inner_fixed;
-          } else {
-            stop = res < tol || it >= I.inner_max;
-            if (stop && !(res < tol)) status |= SGS_ST_INNER_CAP;
-          }
-          if (!(res == res)) {
-            status |= SGS_ST_NONFINITE;
-            stop = true;
-          }
-          double sd[5] = {wd * t6[1], wd * t6[2], wd * t6[3], wd * t6[4], wd * t6[5]};
+          const float rf = tof(sm.red_tote[0]);
+          int sml = clearly_less(rf, rf, tol2f);
+          float f[5];
 #pragma unroll
-          for (int k = 0; k < 5; k++) sm.svE[k] = w * sm.red_tote[1 + k];
-          bool exists = pfp && sd[0] > 0.0 && sd[0] * sd[4] > sd[1] * sd[1] + sd[2] * sd[2] + sd[3] * sd[3];
-          if (pfp && !exists && relax) exists = relax_target<E>(sm, w, false, sd);
-          sm.ctl = (stop ? 1 : 0) | (exists ? 2 : 0);
+          for (int k = 0; k < 5; k++) {
+            const E sk = w * sm.red_tote[1 + k];
+            sm.svE[k] = sk;
+            f[k] = tof(sk);
+          }
+          int ex = pfp ? clearly_exists(f[0], f[1], f[2], f[3], f[4]) : 0;
+          if (sml < 0 || ex < 0 || (pfp && relax && ex == 0)) {  // in FP64
+            const double res = sqrt(wd * t6[0]);
+            sml = res < I.inner_tol;
+            if (!(res == res)) sml = 2;
+            double sd[5] = {wd * t6[1], wd * t6[2], wd * t6[3], wd * t6[4], wd * t6[5]};
+            bool exists = pfp && sd[0] > 0.0 && sd[0] * sd[4] > sd[1] * sd[1] + sd[2] * sd[2] + sd[3] * sd[3];
+            if (pfp && !exists && relax) exists = relax_target<E>(sm, w, sd);
+            ex = exists;
+          }
+          sm.ctl = (decide(sml) ? 1 : 0) | (ex ? 2 : 0);
         }
         __syncthreads();
       }
@@ -729,7 +723,7 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
           if (tid < 5) sm.thp[tid] = sm.thg[tid];
           __syncthreads();
           // the last evaluation is M[g]'s: reused as the first one of step 1
-          int n1 = newton_cta<E>(sm, N, w, 1, sv, sm.thp, L, ntol, I.newton_max, true);
+          int n1 = newton_cta<E>(sm, N, w, true, sv, sm.thp, L, ntol, I.newton_max, true);
           c_solves++;
           if (n1 >= 0) {
             c_newton += n1;
@@ -743,16 +737,14 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
       E (*Eu)[kMaxN] = used ? sm.Ep : sm.Eg;
       // moments of M+: step 1's last evaluation is at M+; M[g] has the moments of g
       E momP[5];
-      if (!lowp) {
-        if (used) {
-          float Aa[15];
-          moments_from_sums<E>(sm.S[0], sm.S[1], sm.S[2], momP, Aa);
+      if (used) {
+        float Aa[15];
+        moments_from_sums<E>(sm.S[0], sm.S[1], sm.S[2], momP, Aa);
 #pragma unroll
-          for (int k = 0; k < 5; k++) momP[k] = w * momP[k];
-        } else {
+        for (int k = 0; k < 5; k++) momP[k] = w * momP[k];
+      } else {
 #pragma unroll
-          for (int k = 0; k < 5; k++) momP[k] = momg[k];
-        }
+        for (int k = 0; k < 5; k++) momP[k] = momg[k];
       }
 
       // ---- step 2 (eq. (25)) and the moments of the new iterate
@@ -769,7 +761,7 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
         }
       }
       // keep the factors of M+ in sm.Ep (the reduction below orders this before solve_mg)
-      if (!lowp && !used && tid < 3 * kMaxN) sm.Ep[tid / kMaxN][tid % kMaxN] = sm.Eg[tid / kMaxN][tid % kMaxN];
+      if (!used && tid < 3 * kMaxN) sm.Ep[tid / kMaxN][tid % kMaxN] = sm.Eg[tid / kMaxN][tid % kMaxN];
       E m5[5] = {c0, v1 * c0, v2 * c0, c3, vq12 * c0 + c4};
       double t5[5];
       cluster_reduce<5, E>(m5, t5, sm, buf, cl, CS);
@@ -781,19 +773,22 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
       int n2 = solve_mg<E>(sm, N, w, mm, used ? sm.thp : sm.thg, eval_at_start, L, ntol, I.newton_max, status);
       if (n2 > 0) c_newton += n2;
       c_solves++;
-      if (!lowp) {
-        // ---- residual and step-1 target of the new iterate from the step-2 identity
-        derived_sums<E>(sm);
-        // warp 0 decides; its lanes form the five components of the step-1 target and the
-        // residual norm concurrently (a serial chain of double-float operations otherwise)
-        if (tid < 32) {
-          const int lane = tid;
-          E sk = zero;
-          if (lane < 5) {
-            const E mwk = moment_k<E>(sm.S1w, sm.S[1], sm.S[2], lane);  // sum phi (|v1|/dx) M[g]
-            sk = w * mwk - Acoef * pick5<E>(momP, lane) + Acoef * pick5<E>(mm, lane);
-            sm.svE[lane] = sk;
-          }
+      // ---- residual and step-1 target of the new iterate from the step-2 identity
+      derived_sums<E>(sm);
+      // warp 0 decides; its lanes form the five components of the step-1 target
+      if (tid < 32) {
+        const int lane = tid;
+        const E mwk = lane_moment<E>(sm.S1w, sm.S[1], sm.S[2], lane);  // sum phi (|v1|/dx) M[g]
+        const E sk = w * mwk - Acoef * pick5<E>(momP, lane) + Acoef * pick5<E>(mm, lane);
+        if (lane < 5) sm.svE[lane] = sk;
+        float mag;
+        const float nf = derived_norm2_f32(sm, mag);
+        int sml = clearly_less(nf, mag, limf);
+        float f[5];
+#pragma unroll
+        for (int k = 0; k < 5; k++) f[k] = shfl_i(tof(sk), k);
+        int ex = pfp ? clearly_exists(f[0], f[1], f[2], f[3], f[4]) : 0;
+        if (sml < 0 || ex < 0 || (pfp && relax && ex == 0)) {  // in FP64, from the full sums
           const double sdk = tod(sk);
           double nrm = lane == 5 ? tod(derived_norm2<E>(sm)) : 0.0;
           double sd[5];
@@ -802,34 +797,25 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
           nrm = __shfl_sync(0xffffffffu, nrm, 5);
           __syncwarp();  // the lanes' sm.svE before lane 0 may replace them (relaxed step 1)
           if (lane == 0) {
-            const double Ad = tod(Acoef);
-            const double res = fabs(Ad) * sqrt(wd * nrm);
-            bool stop;
-            if (I.inner_fixed > 0) {
-              stop = it >= I.inner_fixed;
-            } else {
-              stop = res < I.inner_tol || it >= I.inner_max;
-              if (stop && !(res < I.inner_tol)) status |= SGS_ST_INNER_CAP;
-            }
-            if (!(res == res)) {
-              status |= SGS_ST_NONFINITE;
-              stop = true;
-            }
+            const double res = fabs(tod(Acoef)) * sqrt(wd * nrm);
+            sml = res < I.inner_tol;
+            if (!(res == res)) sml = 2;
             bool exists = pfp && sd[0] > 0.0 && sd[0] * sd[4] > sd[1] * sd[1] + sd[2] * sd[2] + sd[3] * sd[3];
-            if (pfp && !exists && relax) exists = relax_target<E>(sm, w, false, sd);
-            sm.ctl = (stop ? 1 : 0) | (exists ? 2 : 0);
+            if (pfp && !exists && relax) exists = relax_target<E>(sm, w, sd);
+            ex = exists;
           }
         }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < 5; k++) momg[k] = mm[k];
-        derived = true;
+        if (lane == 0) sm.ctl = (decide(sml) ? 1 : 0) | (ex ? 2 : 0);
       }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < 5; k++) momg[k] = mm[k];
+      derived = true;
     }
 
     if (own) {
 #pragma unroll
-      for (int t = 0; t < EPT; t++) fj[t] = tod(g[t]);
+      for (int t = 0; t < EPT; t++) fj[t] = widen(g[t]);
     }
     c_inner += it;
     // the next visit's first reduction is a cluster barrier: every CTA has finished this
