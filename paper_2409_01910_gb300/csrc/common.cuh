@@ -150,22 +150,24 @@ __device__ __forceinline__ E cvt(double x);
 template <>
 __device__ __forceinline__ double cvt<double>(double x) { return x; }
 template <>
-__device__ __forceinline__ float cvt<float>(double x) { return (float)x; }
-template <>
 __device__ __forceinline__ dfloat cvt<dfloat>(double x) {
   return df_split(x);
 }
 __device__ __forceinline__ double tod(double x) { return x; }
-__device__ __forceinline__ double tod(float x) { return (double)x; }
 __device__ __forceinline__ double tod(dfloat x) { return (double)x.hi + (double)x.lo; }
 __device__ __forceinline__ float tof(double x) { return (float)x; }
 __device__ __forceinline__ float tof(float x) { return x; }
 __device__ __forceinline__ float tof(dfloat x) { return x.hi; }
 
-// exp in the precision of E without leaving it
-__device__ __forceinline__ double exp_in(double x) { return exp(x); }
-__device__ __forceinline__ float exp_in(float x) { return expf(x); }
-__device__ __forceinline__ dfloat exp_in(dfloat x) { return df_exp(x); }
+// The double of an FP32 number, and of a double-float, with the bits of the conversion: a normal
+// number is widened by integer operations (a conversion holds the FP64 unit for 101 cycles).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)x;  // subnormal, infinite, NaN
+  const unsigned hi = (u & 0x80000000u) | (m == 0u ? 0u : (m >> 3) + 0x38000000u);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(dfloat x) { return widen(x.hi) + widen(x.lo); }
 
 __device__ __forceinline__ double shfl_x(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ float shfl_x(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }

@@ -53,6 +53,7 @@ struct SweepSmem {
   E ef[3][kMaxN];           // factors of the Maxwellian that the next pass over the nodes reads
   E W[4][3][kMaxN];         // unit wall Maxwellians
   E etab[64];               // 2^(j/64)
+  double vm[2][kMaxN];      // 2-D FP64: node numbers m and m^2
   E rows[2][kRows][4];     // Newton evaluations, double-buffered: sums of powers 0-2, one row per warp
   E warp_part[kRed][8];
   E part[2][16][kRed];      // partial sums of every CTA of the cluster
@@ -79,6 +80,21 @@ template <>
 struct Node<dfloat> {
   typedef float M;
 };
+// Node i and its square as M. An int -> FP64 conversion holds the FP64 unit of a scheduler for 101
+// cycles (a multiply: 64), so the 2-D FP64 passes, two fifths of a visit there, read both from a
+// table (40 x 40 cells, 20 velocities, BGK: 32.35 -> 31.59 ms). In 1-D FP64 the table costs the
+// Newton loop more than the passes gain (16 cells, 16 velocities: 6.38 -> 6.62 ms), and in FP32 a
+// conversion is as cheap as a load.
+template <typename M, bool TWO_D>
+__device__ __forceinline__ M node_m(const double (&vm)[2][kMaxN], int i, int N) {
+  if constexpr (TWO_D && sizeof(M) == 8) return vm[0][i];
+  return (M)(i + 1 - N / 2);
+}
+template <typename M, bool TWO_D>
+__device__ __forceinline__ M node_q(const double (&vm)[2][kMaxN], int i, M m) {
+  if constexpr (TWO_D && sizeof(M) == 8) return vm[1][i];
+  return m * m;
+}
 // Double-float sums and products without the final renormalisation: (hi, lo) whose halves may
 // overlap by a few bits. In a chain of additions the leading parts then depend on each other
 // through one FP32 addition only, and an addition takes 8 operations instead of 11; norm()
@@ -546,6 +562,9 @@ __device__ __forceinline__ void scan_tables(SweepSmem<E>& sm, const InstDev& I, 
     const double v = tid < N ? node(tid, N, dv) : 0.0;
     sm.c1e[tid] = cvt<E>(fabs(v) * I.inv_dx);
     sm.c2e[tid] = TWO_D ? cvt<E>(fabs(v) * I.inv_dy) : cvt<E>(0.0);
+    const double m = tid + 1 - N / 2;
+    sm.vm[0][tid] = m;
+    sm.vm[1][tid] = m * m;
   }
 #pragma unroll 1
   for (int t = tid; t < (TWO_D ? 4 : 2) * 3 * kMaxN; t += blockDim.x)
@@ -624,7 +643,7 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
       const int i1 = pen / N, i2 = pen - i1 * N;
       const int e0 = run * R;
       const int sgn1 = i1 + 1 - N / 2, sgn2 = i2 + 1 - N / 2;  // v1, v2 in units of dv
-      const M v1 = (M)sgn1, v2 = (M)sgn2;
+      const M v1 = node_m<M, TWO_D>(sm.vm, i1, N), v2 = node_m<M, TWO_D>(sm.vm, i2, N);
       double x[R];
       load_run(io.f + e0, x);
       if (pass == 0) {
@@ -678,7 +697,7 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
 #pragma unroll
         for (int t = 0; t < R; t++) {
           const int i3 = i30 + t;
-          const M v3 = (M)(i3 + 1 - N / 2), vq3 = v3 * v3;
+          const M v3 = node_m<M, TWO_D>(sm.vm, i3, N), vq3 = node_q<M, TWO_D>(sm.vm, i3, v3);
           const E g = cvt<E>(x[t]);
           E r = -umul(cvt<E>(pv[t]), inv_eps);
           if (sgn1 != 0) r = uadd(r, -umul(c1, cvt<E>(u1[t])));
@@ -1015,10 +1034,10 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
 #pragma unroll 1
             for (int i2 = wid; i2 < N; i2 += nev) {
               const E t = norm(umul(den2[i2 * N + lane], sm.ef[1][i2]));
-              const M m2 = (M)(i2 + 1 - N / 2);
+              const M m2 = node_m<M, TWO_D>(sm.vm, i2, N);
               w0 = uadd(w0, t);
               w1 = uadd_mul(w1, t, m2);
-              w2 = uadd_mul(w2, t, m2 * m2);
+              w2 = uadd_mul(w2, t, node_q<M, TWO_D>(sm.vm, i2, m2));
             }
           }
           const E e1 = lane < N ? sm.ef[0][lane] : zero;

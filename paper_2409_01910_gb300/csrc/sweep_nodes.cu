@@ -62,16 +62,6 @@ struct NodesSmem {
   int nret;            // Newton result, for the warps that do not evaluate
 };
 
-// The double of an FP32 number, and of a double-float, with the bits of the conversion: a normal
-// number is widened by integer operations (a conversion holds the FP64 unit for 101 cycles).
-__device__ __forceinline__ double widen(float x) {
-  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
-  if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)x;  // subnormal, infinite, NaN
-  const unsigned hi = (u & 0x80000000u) | (m == 0u ? 0u : (m >> 3) + 0x38000000u);
-  return __hiloint2double((int)hi, (int)(u << 29));
-}
-__device__ __forceinline__ double widen(dfloat x) { return widen(x.hi) + widen(x.lo); }
-
 __device__ __forceinline__ float shfl_i(float v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
 __device__ __forceinline__ dfloat shfl_i(dfloat v, int lane) { return {shfl_i(v.hi, lane), shfl_i(v.lo, lane)}; }
 
@@ -167,7 +157,7 @@ __device__ __noinline__ void eval_cta(NodesSmem<E>& sm, int N) {
     if (lane < N) {
       E x = sm.thE[1 + d] * sm.vv[lane] - sm.thE[4] * sm.vq[lane];
       if (d == 0) x += sm.thE[0];
-      e = exp_in(x);
+      e = df_exp(x);
     }
     if (wid < 3) sm.ef[d][lane] = e;
     if (wid == 3) e = e * sm.c1e[lane];
@@ -271,7 +261,7 @@ __device__ __forceinline__ void eval_warp(NodesSmem<E>& sm, int N, E thl, int wi
   if (lane < N) {
     E x = b * sm.vv[lane] - g * sm.vq[lane];
     if (d == 0) x += al;
-    e = exp_in(x);
+    e = df_exp(x);
   }
   if (wid < 3) sm.ef[d][lane] = e;
   if (wid == 3) e = e * sm.c1e[lane];
