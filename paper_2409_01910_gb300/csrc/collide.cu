@@ -40,33 +40,28 @@ __device__ inline double maxwell_factor(const double* th, int d, int i, int N, d
 // residual grows; stop one step after the exponent change |da| + L sum|db| + L^2 |dg| falls below
 // tol) follows the discrete conservation equations directly.
 //
-// Called by one full warp; lane i < N handles node i. All lanes return the same result. The 15
-// sums are reduced together: a lane keeps half of its values in each step and hands the other
-// half to its partner (16 additions instead of 75 of the scarce FP64 pipe, the same pairs).
+// Called by four warps (wt = 0-3), each on its own scheduler: an FP64 instruction takes a scheduler
+// 64 cycles, in a chain or not, so the solve is bound by the number of them in its longest chain.
+// Warp d < 3 evaluates dimension d (lane i: node i), warp 3 the factor exp(alpha); after one
+// barrier each warp combines the sums, lane k forming component k of the moments, residual and
+// exponents (about 45 FP64 instructions an evaluation, 175 on one warp: 5.7 us), and takes the same
+// decisions. FP64 expressions that the compiler may contract either way name their rounded product.
 // ---------------------------------------------------------------------------------------
-struct MaxwEval {
-  double F[5];  // moments of M minus the target
-  float A[15];  // upper triangle of sum w M phi phi^T (row-major, i <= j): Newton direction only
-  double fn;    // max |F_i| / |target_0|
+struct NewtonSmem {
+  double S[2][3][5], ea[2];  // sums of an evaluation and its exp(alpha), double-buffered
+  float Sf[2][3][5];
 };
 
-__device__ inline void maxw_eval(int N, double dv, double w, const double* target, const double* th, MaxwEval& out) {
-  const int lane = threadIdx.x & 31;
-  double v[16];
-  const double vd = node(lane < N ? lane : 0, N, dv), v2 = vd * vd;
-#pragma unroll
-  for (int d = 0; d < 3; d++) {
-    const double x = lane < N ? exp(th[1 + d] * vd - th[4] * vd * vd) : 0.0;
-    v[5 * d + 0] = x;
-    v[5 * d + 1] = x * vd;
-    v[5 * d + 2] = v[5 * d + 1] * vd;
-    v[5 * d + 3] = v[5 * d + 2] * vd;
-    v[5 * d + 4] = v[5 * d + 2] * v2;
-  }
-  v[15] = 0.0;
+__device__ __forceinline__ void newton_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// Sums over the warp of five values per lane, lane l returning the total of value l / 4: in the first
+// three steps a lane keeps half of its values and hands over the other half (the pairs of a
+// butterfly over all of them with 9 additions instead of 25).
+__device__ __forceinline__ double warp_sums5(const double (&x)[5], int lane) {
+  double v[8] = {x[0], x[1], x[2], x[3], x[4], 0.0, 0.0, 0.0};
   int o = 16;
 #pragma unroll
-  for (int h = 8; h >= 1; h >>= 1, o >>= 1) {
+  for (int h = 4; h >= 1; h >>= 1, o >>= 1) {
     const bool up = (lane & o) != 0;
 #pragma unroll
     for (int q = 0; q < h; q++) {
@@ -74,31 +69,64 @@ __device__ inline void maxw_eval(int N, double dv, double w, const double* targe
       v[q] = keep + shfl_x(send, o);
     }
   }
-  const double t = v[0] + shfl_x(v[0], 1);  // total of value lane / 2
-  const float tf = (float)t;
-  double s[15];
-  float f[15];
-#pragma unroll
-  for (int q = 0; q < 15; q++) {
-    s[q] = __shfl_sync(0xffffffffu, t, 2 * q);
-    f[q] = __shfl_sync(0xffffffffu, tf, 2 * q);
+  v[0] += shfl_x(v[0], 2);
+  return v[0] + shfl_x(v[0], 1);
+}
+
+// Moments of M at the exponents th (lane k: component k) minus the target (lane k: tl): Ff on every
+// lane, the Jacobian A (upper triangle of sum w M phi phi^T, row-major, i <= j: it only sets the
+// direction) and the largest |F|.
+__device__ __forceinline__ void maxw_eval(NewtonSmem& sm, int N, double dv, double w, double tl, double th, int wt,
+                                          int buf, float (&Ff)[5], float (&A)[15], double& amax) {
+  const int lane = threadIdx.x & 31;
+  if (wt < 3) {
+    const double vd = node(lane < N ? lane : 0, N, dv), v2 = vd * vd;
+    const double b = __shfl_sync(0xffffffffu, th, 1 + wt), g = __shfl_sync(0xffffffffu, th, 4);
+    const double x = lane < N ? exp(b * vd - g * vd * vd) : 0.0;
+    double v[5];
+    v[0] = x;
+    v[1] = x * vd;
+    v[2] = v[1] * vd;
+    v[3] = v[2] * vd;
+    v[4] = v[2] * v2;
+    const double t = warp_sums5(v, lane);
+    const float tf = (float)t;
+    if ((lane & 3) == 0 && lane < 20) {
+      sm.S[buf][wt][lane >> 2] = t;
+      sm.Sf[buf][wt][lane >> 2] = tf;
+    }
+  } else {
+    const double ea = exp(__shfl_sync(0xffffffffu, th, 0));
+    if (lane == 0) sm.ea[buf] = ea;
   }
-  const double ea = exp(th[0]);
-  const double *S1 = s, *S2 = s + 5, *S3 = s + 10;
-  const double c = w * ea;
-  // sums of phi_i M over the grid, from the 1-D sums
-  const double s23 = S2[0] * S3[0];
-  const double mom[5] = {S1[0] * s23, S1[1] * s23, S1[0] * (S2[1] * S3[0]), S1[0] * (S2[0] * S3[1]),
-                         S1[2] * s23 + S1[0] * (S2[2] * S3[0] + S2[0] * S3[2])};
-  double amax = 0.0;
+  newton_bar();
+  const double *S1 = sm.S[buf][0], *S2 = sm.S[buf][1], *S3 = sm.S[buf][2];
+  const double c = w * sm.ea[buf];
+  // lane k: sum of phi_k M over the grid, from the 1-D sums (lanes 5 and 6 form parts of the last one)
+  const int i = lane == 1 ? 1 : (lane == 4 ? 2 : 0), j = lane == 2 ? 1 : (lane == 5 ? 2 : 0),
+            l = lane == 3 ? 1 : (lane == 6 ? 2 : 0);
+  double u = __dmul_rn(S2[j], S3[l]);
+  const double u6 = __shfl_sync(0xffffffffu, u, 6);
+  if (lane == 5) u = __fma_rn(S2[2], S3[0], u6);
+  double m = __dmul_rn(S1[i], u);
+  const double m5 = __shfl_sync(0xffffffffu, m, 5);
+  if (lane == 4) m = __fma_rn(S1[2], u, m5);
+  const double F = __fma_rn(c, m, -tl);
+  const float Fl = (float)F;
 #pragma unroll
-  for (int i = 0; i < 5; i++) {
-    out.F[i] = c * mom[i] - target[i];
-    amax = fmax(amax, fabs(out.F[i]));
+  for (int k = 0; k < 5; k++) Ff[k] = __shfl_sync(0xffffffffu, Fl, k);
+  // largest |F| of lanes 0-4 as an integer (non-negative doubles order like their bits); a NaN drops
+  // out, as it does from fmax
+  unsigned long long bits = (unsigned long long)__double_as_longlong(F) & 0x7fffffffffffffffull;
+  if (lane > 4 || bits > 0x7ff0000000000000ull) bits = 0;
+#pragma unroll
+  for (int o = 4; o >= 1; o >>= 1) {
+    const unsigned long long other = __shfl_xor_sync(0xffffffffu, bits, o);
+    bits = other > bits ? other : bits;
   }
-  out.fn = amax / fabs(target[0]);
-  // Jacobian entries in FP32: they only set the Newton direction
-  const float *f1 = f, *f2 = f + 5, *f3 = f + 10;
+  amax = __longlong_as_double((long long)__shfl_sync(0xffffffffu, bits, 0));
+  // Jacobian entries in FP32
+  const float *f1 = sm.Sf[buf][0], *f2 = sm.Sf[buf][1], *f3 = sm.Sf[buf][2];
   float q11 = f1[2] * f2[0] * f3[0], q22 = f1[0] * f2[2] * f3[0], q33 = f1[0] * f2[0] * f3[2];
   float q12 = f1[1] * f2[1] * f3[0], q13 = f1[1] * f2[0] * f3[1], q23 = f1[0] * f2[1] * f3[1];
   float c1 = f1[3] * f2[0] * f3[0] + f1[1] * f2[2] * f3[0] + f1[1] * f2[0] * f3[2];
@@ -106,43 +134,60 @@ __device__ inline void maxw_eval(int N, double dv, double w, const double* targe
   float c3 = f1[2] * f2[0] * f3[1] + f1[0] * f2[2] * f3[1] + f1[0] * f2[0] * f3[3];
   float e4 = f1[4] * f2[0] * f3[0] + f1[0] * f2[4] * f3[0] + f1[0] * f2[0] * f3[4] +
              2.0f * (f1[2] * f2[2] * f3[0] + f1[2] * f2[0] * f3[2] + f1[0] * f2[2] * f3[2]);
-  float cf = (float)c;
-  float A[15] = {f1[0] * f2[0] * f3[0], f1[1] * f2[0] * f3[0], f1[0] * f2[1] * f3[0], f1[0] * f2[0] * f3[1],
-                 q11 + q22 + q33, q11, q12, q13, c1, q22, q23, c2, q33, c3, e4};
+  const float cf = (float)c;
+  const float B[15] = {f1[0] * f2[0] * f3[0], f1[1] * f2[0] * f3[0], f1[0] * f2[1] * f3[0], f1[0] * f2[0] * f3[1],
+                       q11 + q22 + q33, q11, q12, q13, c1, q22, q23, c2, q33, c3, e4};
 #pragma unroll
-  for (int i = 0; i < 15; i++) out.A[i] = cf * A[i];
+  for (int q = 0; q < 15; q++) A[q] = cf * B[q];
 }
 
-// Newton for the discrete Maxwellian from the guess in th. The residual F is evaluated in FP64 and
-// the direction from the FP32 factorisation (inexact Newton: the root is the one of F). The step
-// is halved while the scaled residual grows; the iteration stops right after a step whose
-// exponent change |da| + L sum|db| + L^2 |dg| is below tol.
-__device__ inline int maxwellian_newton(int N, double dv, double w, const double* target, double* th, double tol,
-                                        int maxit) {
+// Newton for the discrete Maxwellian from the guess in th (lane k: component k). The residual F is
+// evaluated in FP64 and the direction from the FP32 factorisation (inexact Newton: the root is the
+// one of F). The step is halved while the scaled residual max |F| / rho grows; the iteration stops
+// right after a step whose exponent change |da| + L sum|db| + L^2 |dg| is below tol. Decisions are
+// taken without FP64 where that leaves no doubt.
+__device__ __forceinline__ int maxwellian_newton(NewtonSmem& sm, int N, double dv, double w, double tl, double& th,
+                                                 double tol, int maxit, int wt) {
+  const int kl = min((int)(threadIdx.x & 31), 4);
   const double L = node(N - 1, N, dv);
-  MaxwEval ev;
-  maxw_eval(N, dv, w, target, th, ev);
+  const double rho = fabs(__shfl_sync(0xffffffffu, tl, 0));
+  const float Lf = (float)L, tolf = (float)tol;
+  float Ff[5], A[15];
+  double amax;
+  int buf = 0;
+  maxw_eval(sm, N, dv, w, tl, th, wt, buf, Ff, A, amax);
   for (int it = 0; it < maxit; it++) {
-    float y[5], Ff[5];
+    float y[5];
+    if (!chol5_solve(A, Ff, y)) return -1;
+    float yl = y[0];
 #pragma unroll
-    for (int i = 0; i < 5; i++) Ff[i] = (float)ev.F[i];
-    if (!chol5_solve(ev.A, Ff, y)) return -1;
-    double d[5] = {-(double)y[0], -(double)y[1], -(double)y[2], -(double)y[3], (double)y[4]};  // -D A^{-1} F
-    double lam = 1.0;
-    double fn = ev.fn;
-    double tt[5];
+    for (int k = 1; k < 5; k++)
+      if (k == kl) yl = y[k];
+    const double d = widen(kl == 4 ? yl : -yl);  // -D A^{-1} F
+    const double before = amax;
+    double lam = 1.0, tt;
+    float lamf = 1.0f;
     for (int hv = 0; hv < 40; hv++) {
-#pragma unroll
-      for (int i = 0; i < 5; i++) tt[i] = th[i] + lam * d[i];
-      maxw_eval(N, dv, w, target, tt, ev);
-      if (ev.fn == ev.fn && (ev.fn <= fn || ev.fn <= 1e-10)) break;
+      tt = __fma_rn(lam, d, th);
+      buf ^= 1;
+      maxw_eval(sm, N, dv, w, tl, tt, wt, buf, Ff, A, amax);
+      if (amax <= before || amax < 0.99e-10 * rho) break;  // (division by rho is monotone)
+      const double fn = amax / rho, f0 = before / rho;
+      if (fn == fn && (fn <= f0 || fn <= 1e-10)) break;
       lam *= 0.5;
+      lamf *= 0.5f;
     }
-#pragma unroll
-    for (int i = 0; i < 5; i++) th[i] = tt[i];
-    double step = lam * (fabs(d[0]) + L * (fabs(d[1]) + fabs(d[2]) + fabs(d[3])) + L * L * fabs(d[4]));
-    if (!(step == step)) return -1;
-    if (step <= tol) return it + 1;
+    th = tt;
+    const float sf = lamf * (fabsf(y[0]) + Lf * (fabsf(y[1]) + fabsf(y[2]) + fabsf(y[3])) + Lf * Lf * fabsf(y[4]));
+    bool done = sf < tolf;
+    if (!(tolf > 1e-30f && fabsf(sf - tolf) > 1e-4f * (sf + tolf))) {
+      const double step =
+          lam * (fabs((double)y[0]) + L * (fabs((double)y[1]) + fabs((double)y[2]) + fabs((double)y[3])) +
+                 L * L * fabs((double)y[4]));
+      if (!(step == step)) return -1;
+      done = step <= tol;
+    }
+    if (done) return it + 1;
   }
   return -1;
 }
@@ -152,20 +197,27 @@ __device__ inline int maxwellian_newton(int N, double dv, double w, const double
 // factors of the Maxwellian (E_d[i], E_1 with exp(alpha)) that the transforms read.
 //
 // The sums are bound by the FP64 pipe of one SM (8 instructions a node: 85 us for 32^3 nodes). For
-// a call of few cells the eight warps of a cell are therefore eight CTAs of a cluster (SPLIT), on
-// as many SMs; every warp adds the same nodes in the same order in both forms, so the results
-// are the same bits. 32 cells of 32^3: 132 -> 89 us, 8 cells of 8^3: 57 -> 44 us (the rest is
-// Newton, on one warp: an FP64 instruction takes a scheduler 64 cycles, in a chain or not).
+// a call of few cells the eight warps of a cell are therefore two CTAs of a cluster (SPLIT), each
+// warp on a scheduler of its own; every warp adds the same nodes in the same order in both forms,
+// so the results are the same bits. What follows, the guess and Newton, runs on four warps of
+// the first CTA. 8 cells of 8^3: 57 us in one CTA, 44 with Newton on one warp of a split cell, 25
+// now; 64 cells of 32^3: 89 (32 cells) with one warp, 75 now. (Eight CTAs of four warps a
+// cell don't fit side by side on the chip: 128 cells of 32^3 took 164 us instead of 98.)
 // ---------------------------------------------------------------------------------------
 template <bool SPLIT>
-__global__ void __launch_bounds__(SPLIT ? 32 : 256) k_moments(const double* __restrict__ f, CellTables ct, int N,
+constexpr int kMomentsThreads = SPLIT ? 128 : 256;  // Newton's barrier needs four warps at least
+template <bool SPLIT>
+__global__ void __launch_bounds__(kMomentsThreads<SPLIT>) k_moments(const double* __restrict__ f, CellTables ct, int N,
                                                                double dv, double newton_tol, int newton_max,
                                                                double* __restrict__ theta, double* __restrict__ nu,
                                                                double* __restrict__ efac, Counters* cnt) {
   __shared__ double vv[kMaxN];
   __shared__ double part[8][5];
-  const int wid = SPLIT ? (int)(blockIdx.x & 7) : (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int c = SPLIT ? blockIdx.x >> 3 : blockIdx.x;
+  __shared__ NewtonSmem sm;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = SPLIT ? (int)(blockIdx.x & 1) : 0;  // in the cluster: a cluster is one cell
+  const int wid = 4 * rank + warp;                     // part of the sums
+  const int c = SPLIT ? blockIdx.x >> 1 : blockIdx.x;
   if (!cell_active(ct.active, ct.cell_inst, c)) return;  // whole cluster, uniformly
   int K = N * N * N;
   const double* fc = f + ct.cell_off[c];
@@ -184,33 +236,43 @@ __global__ void __launch_bounds__(SPLIT ? 32 : 256) k_moments(const double* __re
     s[3] += x * d;
     s[4] += x * (a * a + b * b + d * d);
   }
-  warp_allsum<5>(s);
+  const double sum = warp_sums5(s, lane);
+  const bool holds = (lane & 3) == 0 && lane < 20;
   if (SPLIT) {
     cg::cluster_group cl = cg::this_cluster();
     cl.barrier_wait();
-    if (lane == 0) {
-      double* p = cl.map_shared_rank(&part[wid][0], 0);  // rank = wid: a cluster is one cell
-      for (int q = 0; q < 5; q++) p[q] = s[q];
-    }
+    if (holds) cl.map_shared_rank(&part[wid][0], 0)[lane >> 2] = sum;
     cl.sync();
-    if (wid != 0) return;  // only its own writes were remote, and they have landed
+    if (rank != 0) return;  // only its own writes were remote, and they have landed
   } else {
-    if (lane == 0)
-      for (int q = 0; q < 5; q++) part[wid][q] = s[q];
+    if (holds) part[wid][lane >> 2] = sum;
     __syncthreads();
-    if (wid != 0) return;
+    if (warp >= 4) return;
   }
-  double w = dv * dv * dv;
-  double m[5];
-  for (int q = 0; q < 5; q++) {
-    double t = 0.0;
-    for (int k = 0; k < 8; k++) t += part[k][q];
-    m[q] = w * t;
-  }
+  const double w = dv * dv * dv;
+  const int kl = min(lane, 4);
+  double t = 0.0;
+  for (int q = 0; q < 8; q++) t += part[q][kl];
+  const double ml = w * t;  // lane k: moment k
+  double m[5], th[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+  for (int q = 0; q < 5; q++) m[q] = __shfl_sync(0xffffffffu, ml, q);
   const InstDev& I = ct.inst[ct.cell_inst[c]];
-  double th[5] = {0, 0, 0, 0, 0};
   int it = -1;
-  if (continuum_guess<double>(m, th)) it = maxwellian_newton(N, dv, w, m, th, newton_tol, newton_max);
+  double thl = 0.0;  // lane k: exponent k
+  if (continuum_guess<double>(m, th)) {
+    thl = th[0];
+#pragma unroll
+    for (int q = 1; q < 5; q++)
+      if (q == kl) thl = th[q];
+    it = maxwellian_newton(sm, N, dv, w, ml, thl, newton_tol, newton_max, warp);
+#pragma unroll
+    for (int q = 0; q < 5; q++) th[q] = __shfl_sync(0xffffffffu, thl, q);
+  }
+  if (warp < 3) {
+    if (lane < N) efac[((long long)c * 3 + warp) * kMaxN + lane] = maxwell_factor(th, warp, lane, N, dv);
+    return;
+  }
   double rho = m[0];
   double T = (m[4] / rho - (m[1] * m[1] + m[2] * m[2] + m[3] * m[3]) / (rho * rho)) / 3.0;
   // penalty frequency of eq. (28): the loss frequency 4 pi b0 rho for Maxwell molecules;
@@ -219,8 +281,8 @@ __global__ void __launch_bounds__(SPLIT ? 32 : 256) k_moments(const double* __re
   // in P (a mean loss frequency lets the explicit remainder grow at large |v|)
   double nuv = 4.0 * kPi * I.b0 * rho;
   if (I.collision == SGS_HARD_SPHERE) nuv *= 2.0 * (N * dv) / (3.0 * sqrt(2.0) + 1.0);
+  if (lane < 5) theta[5 * c + lane] = thl;
   if (lane == 0) {
-    for (int q = 0; q < 5; q++) theta[5 * c + q] = th[q];
     nu[c] = nuv;
     unsigned bits = 0;
     if (it < 0) bits |= SGS_ST_NEWTON_FAIL;
@@ -228,8 +290,6 @@ __global__ void __launch_bounds__(SPLIT ? 32 : 256) k_moments(const double* __re
     if (!(rho == rho) || !(T == T)) bits |= SGS_ST_NONFINITE;
     if (bits) atomicOr(&cnt[ct.cell_inst[c]].status, bits);
   }
-  for (int d = 0; d < 3; d++)
-    if (lane < N) efac[((long long)c * 3 + d) * kMaxN + lane] = maxwell_factor(th, d, lane, N, dv);
 }
 
 // Separable factors of every cell's Maxwellian from theta (one block per cell): of a reference
@@ -1397,22 +1457,22 @@ cudaError_t launch_factors(const double* theta, int C, int N, double dv, double*
 
 // Cells below which the warps of a cell go to different SMs: with more of them the chip's FP64
 // pipes are busy either way, and a CTA per warp only adds launches (128 cells of 32^3: 132 us in
-// one CTA a cell, 122 split).
+// one CTA a cell, 122 with a CTA per warp, 98 with two CTAs).
 constexpr int kMomentsSplit = 304;
 
 cudaError_t launch_moments(const double* f, const CellTables& ct, int C, int N, double dv, double tol, int maxit,
                            double* theta, double* nu, double* efac, Counters* cnt, cudaStream_t st) {
   if (C > kMomentsSplit) {
-    k_moments<false><<<C, 256, 0, st>>>(f, ct, N, dv, tol, maxit, theta, nu, efac, cnt);
+    k_moments<false><<<C, kMomentsThreads<false>, 0, st>>>(f, ct, N, dv, tol, maxit, theta, nu, efac, cnt);
     return cudaGetLastError();
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(8 * C);
-  cfg.blockDim = dim3(32);
+  cfg.gridDim = dim3(2 * C);
+  cfg.blockDim = dim3(kMomentsThreads<true>);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 8;
+  at[0].val.clusterDim.x = 2;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
