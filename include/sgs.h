@@ -348,8 +348,8 @@ int sgs_autotune(sgs_handle* h, double* f, const double* P, int reps, sgs_tuning
  *   sgs_probe_scan: latency of one building block of the persistent scan, in one cluster of
  *     `cluster` CTAs of `threads` threads on the nv^3 grid of [-v_max, v_max]^3, in the scan
  *     arithmetic of a handle of that precision (SGS_FP32: double-float, SGS_FP64: FP64):
- *     mode 0 a cluster reduction of seven values, mode 1 one Newton iteration of the
- *     discrete Maxwellian (evaluation, combination, factorisation), mode 2 the hardware
+ *     mode 0 a cluster reduction of sixteen values, mode 1 one Newton iteration of the
+ *     discrete Maxwellian (evaluation, combination, direction), mode 2 the hardware
  *     cluster barrier alone (one step of the reduction). us_per_op = (time of reps
  *     operations - time of an empty launch) / reps in microseconds. Synchronises the stream. */
 /*   sgs_tc_selftest: check of the tensor-core path of the fast spectral operator (no
