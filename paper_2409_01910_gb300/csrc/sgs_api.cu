@@ -2,6 +2,7 @@
 // Fourier-weight tables, work planning of the spectral sum, workspace layout and the
 // enqueueing of kernels on the caller's stream.
 #include <algorithm>
+#include <cfloat>
 #include <climits>
 #include <cmath>
 #include <cstdio>
@@ -449,7 +450,8 @@ void sgs::fill_inst(const sgs_problem& p, int N, double dv, InstDev& I) {
   I.inv_dx = 1.0 / I.dx;
   I.inv_dy = 1.0 / I.dy;
   I.inv_eps = 1.0 / p.eps;
-  I.tol2_w = p.inner_tol * p.inner_tol / w;
+  // a positive tolerance stays positive (its square may underflow)
+  I.tol2_w = p.inner_tol > 0.0 ? std::max(p.inner_tol * p.inner_tol / w, DBL_MIN) : 0.0;
   for (int s = 0; s < (two_d ? 4 : 2); s++) {
     const sgs_bc& b = p.bc[s];
     const int dn = s < 2 ? 0 : 1;  // normal velocity component of the side

@@ -34,6 +34,8 @@
 // E is the arithmetic of the sums and the Newton residuals: double for the FP64 solver,
 // double-float (two FP32 numbers, FP64-class accuracy, no FP64 instruction on the critical
 // path) for the mixed solver.
+#include <cfloat>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -132,8 +134,6 @@ __device__ __forceinline__ dfloat exponent(dfloat al, dfloat b, dfloat g, float 
   const dfloat t = umul(g, q);
   return uadd(uadd(umul(b, m), dfloat{-t.hi, -t.lo}), al);
 }
-__device__ __forceinline__ bool less(double a, double b) { return a < b; }
-__device__ __forceinline__ bool less(dfloat a, dfloat b) { return (a - b).hi < 0.0f; }
 __device__ __forceinline__ bool is_nan(double a) { return !(a == a); }
 __device__ __forceinline__ bool is_nan(dfloat a) { return !(a.hi == a.hi); }
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -309,6 +309,30 @@ __device__ __forceinline__ void cluster_sum(E (&v)[kRed], SweepSmem<E>& sm, int&
   __syncthreads();
 }
 
+// Binary exponents of the peaks exp(b_d^2 / 4 g) of the three factors of exponents th (the first one
+// carries exp(th0)), and in sum their sum. The squares that form the norm of M+ - M[g] are taken
+// of factors times 2^-k, k fixed for a visit: only the first factor carries exp(alpha), so at a
+// tangential speed U the others peak at exp(U^2 / 2T), whose square leaves FP32 from 9.4 thermal
+// speeds on, and the first one's differences sink below FP32 from about 7. A power of two changes
+// no bit of a norm that was in range.
+__device__ __forceinline__ float norm_scale(float th, int d, int& sum) {
+  const float al = shfl_i(th, 0), q = 0.25f * rcp_approx(shfl_i(th, 4));
+  int kd = 0;
+  sum = 0;
+#pragma unroll
+  for (int t = 0; t < 3; t++) {
+    const float b = shfl_i(th, 1 + t);
+    const float x = 1.44269504f * ((t == 0 ? al : 0.0f) + b * b * q);
+    const int k = (int)rintf(fminf(fmaxf(x, -120.0f), 120.0f));  // (a NaN becomes -120)
+    sum += k;
+    if (t == d) kd = k;
+  }
+  return __int_as_float((127 - kd) << 23);
+}
+// (out of line where E is FP64: in line it takes 0.6 % of an FP64 scan, out of line of a double-float one)
+__device__ __noinline__ float norm_scale(double th, int d, int& sum) { return norm_scale((float)th, d, sum); }
+__device__ __forceinline__ float norm_scale(dfloat th, int d, int& sum) { return norm_scale(th.hi, d, sum); }
+
 // Barrier among the evaluating warps only (hardware barrier 1; __syncthreads uses 0).
 __device__ __forceinline__ void eval_bar(int nwarps) {
   asm volatile("bar.sync 1, %0;" ::"r"(nwarps * 32) : "memory");
@@ -326,7 +350,8 @@ __device__ __forceinline__ void eval_bar(int nwarps) {
 // iteration 0.65 instead of 0.57 us).
 // rows: sum y v^p, p = 0..2, in E; rowsf: the same and p = 3, 4 in FP32, and for rows 0-2 sum
 // (e - p)^2 and sum p (e - p), p the factor of the Maxwellian that step 2 used (for the norm of
-// M+ - M[g]; with p = 0 the first is sum e^2). Returns the lane's factor e.
+// M+ - M[g]; with p = 0 the first is sum e^2), of factors times sc (norm_scale); pf = p sc in
+// FP32. Returns the lane's factor e.
 // ---------------------------------------------------------------------------------------
 template <bool TWO_D>
 __device__ __forceinline__ int row_dim(int role) {  // dimension of a warp's rows
@@ -338,7 +363,7 @@ __device__ __forceinline__ bool two_rows(int role) {
 }
 
 template <typename E, bool TWO_D>
-__device__ __forceinline__ E eval_row(SweepSmem<E>& sm, int N, E th, int role, int lane, int buf, E p) {
+__device__ __forceinline__ E eval_row(SweepSmem<E>& sm, int N, E th, int role, int lane, int buf, E p, float sc) {
   typedef typename Node<E>::M M;
   const E zero = cvt<E>(0.0);
   const int d = row_dim<TWO_D>(role);
@@ -347,7 +372,7 @@ __device__ __forceinline__ E eval_row(SweepSmem<E>& sm, int N, E th, int role, i
   const E b = shfl_i(th, 1 + d), g = shfl_i(th, 4), al = shfl_i(th, 0);
   E e = zero;
   if (lane < N) e = exp_tab(exponent(d == 0 ? al : zero, b, g, m, q), sm.etab);
-  const float df = diff(e, p);
+  const float df = diff(e, p) * sc, pf = tof(p) * sc;
   const E y = role == 3 ? e * sm.c1e[lane] : e;
   const E y2 = umul(y, q);
   const float f3 = tof(y2) * mf, f4 = tof(y2) * qf;
@@ -358,7 +383,7 @@ __device__ __forceinline__ E eval_row(SweepSmem<E>& sm, int N, E th, int role, i
     const E z = e * (TWO_D ? sm.c2e[lane] : sm.den[lane]);
     const E z2 = umul(z, q);
     E s[8] = {y, umul(y, m), y2, zero, z, umul(z, m), z2, zero};
-    float f[8] = {f3, f4, df * df, tof(p) * df, tof(z2) * mf, tof(z2) * qf, 0.0f, 0.0f};
+    float f[8] = {f3, f4, df * df, pf * df, tof(z2) * mf, tof(z2) * qf, 0.0f, 0.0f};
     t = warp_split_sum<8, E>(s, lane);
     tf = warp_split_sum<8, float>(f, lane);
     k = (lane >> 2) & 3;
@@ -367,7 +392,7 @@ __device__ __forceinline__ E eval_row(SweepSmem<E>& sm, int N, E th, int role, i
     if ((lane & 3) != 0) k = kf = -1;
   } else {
     E s[4] = {y, umul(y, m), y2, zero};
-    float f[4] = {f3, f4, df * df, tof(p) * df};
+    float f[4] = {f3, f4, df * df, pf * df};
     t = warp_split_sum<4, E>(s, lane);
     tf = warp_split_sum<4, float>(f, lane);
     if ((lane & 7) != 0) k = kf = -1;
@@ -394,13 +419,13 @@ template <typename E>
 constexpr float kLinear = sizeof(typename Node<E>::M) == 8 ? 1e-8f : 1e-7f;
 template <typename E, bool TWO_D>
 __device__ __forceinline__ E linear_row(SweepSmem<E>& sm, int N, const float (&y)[5], int role, int lane, int buf, E e,
-                                        E p) {
+                                        E p, float sc) {
   const int d = row_dim<TWO_D>(role);
   const float yd = d == 0 ? y[1] : (d == 1 ? y[2] : y[3]), ya = d == 0 ? y[0] : 0.0f;
   const float m = (float)(lane + 1 - N / 2);
   e = addf(e, -tof(e) * (ya + m * (yd + m * y[4])));
-  const float df = diff(e, p);
-  float f[2] = {df * df, tof(p) * df};
+  const float df = diff(e, p) * sc;
+  float f[2] = {df * df, tof(p) * sc * df};
   const float t = warp_split_sum<2, float>(f, lane);
   // lanes 0-4: the warp's own row, lanes 8-12: row 4
   const int k = lane & 7, row = lane < 8 ? role : 4;
@@ -606,9 +631,12 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
   if (team) th = cvt<E>(io.theta[kl]) * cvt<E>(kl == 0 ? 1.0 : (kl < 4 ? a.dv : a.dv * a.dv));
   int cur = 0;  // buffer of the latest evaluation
   E e = zero;   // the lane's factor in it (roles 0-2)
+  int ksum = 0;
+  float sc = 1.0f;
+  if (team) sc = norm_scale(th, row_dim<TWO_D>(wid), ksum);
   if (!TWO_D) __syncthreads();  // sm.den before role 4 reads it
   if (team) {
-    e = eval_row<E, TWO_D>(sm, N, th, wid, lane, cur, zero);
+    e = eval_row<E, TWO_D>(sm, N, th, wid, lane, cur, zero, sc);
     if (wid < 3) sm.ef[wid][lane] = e;
   }
   __syncthreads();
@@ -758,8 +786,9 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
     // there, a further step could only confirm it
     constexpr float ftol = 1e-13f;
     const bool pfp = I.inner_method != SGS_FP, relax = I.inner_method == SGS_PFP_RELAX;
-    const E tol2 = cvt<E>(I.tol2_w);  // inner_tol^2 / w
-    const float tol2f = tof(tol2);
+    // inner_tol^2 / w in the units of the scaled norm; a positive tolerance stays positive
+    const double tol2 = I.tol2_w;
+    const float tol2f = tol2 > 0.0 ? fmaxf((float)(tol2 * __hiloint2double((1023 - 2 * ksum) << 20, 0)), FLT_MIN) : 0.0f;
     const int inner_fixed = I.inner_fixed, inner_max = I.inner_max, newton_max = I.newton_max;
     int it = 0;
     res2 = sm.tot[15];
@@ -800,7 +829,7 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
           asm volatile("" : "+r"(have), "+r"(itn), "+r"(hv), "+r"(cur));
           if (!have) {
             cur ^= 1;
-            e = eval_row<E, TWO_D>(sm, N, tr, wid, lane, cur, psub);
+            e = eval_row<E, TWO_D>(sm, N, tr, wid, lane, cur, psub, sc);
             eval_bar(nev);
             moved = 1;
           }
@@ -873,7 +902,7 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
           tr = addf(th, yl);
           if (stepf <= kLinear<E>) {
             cur ^= 1;
-            e = linear_row<E, TWO_D>(sm, N, y, wid, lane, cur, e, psub);
+            e = linear_row<E, TWO_D>(sm, N, y, wid, lane, cur, e, psub, sc);
             eval_bar(nev);
             moved = 1;
             th = tr;
@@ -955,7 +984,7 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
           for (int d = 0; d < 3; d++) QQ[d] = rf[d][5];
           s = mw - tu;
           momg = tgt;
-          small = less(res2, tol2);
+          small = to_store(res2) < tol2;  // in FP64: a double-float ends at 2^-100
           nan = is_nan(res2);
         } else {
           // norm of R = A (M+ - M[g]) and the next step-1 target from the step-2 identity
@@ -992,15 +1021,16 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
         }
         if (stop) break;
         // existence test of step 1 (eq. (26)): s0 s4 > s1^2 + s2^2 + s3^2; where the FP32 values
-        // leave it open, in E
+        // leave it open (the ends of their range among it), in FP64
         const float sf = tof(s);
         const float f0 = shfl_i(sf, 0), f1 = shfl_i(sf, 1), f2 = shfl_i(sf, 2), f3 = shfl_i(sf, 3),
                     f4 = shfl_i(sf, 4);
-        const float pl = f0 * f4, mi = f1 * f1 + f2 * f2 + f3 * f3;
+        const float pl = f0 * f4, mi = f1 * f1 + f2 * f2 + f3 * f3, mag = fabsf(pl) + mi;
         bool exists = pfp && f0 > 0.0f && pl > mi;
-        if (pfp && f0 > 0.0f && fabsf(pl - mi) <= 1e-5f * (fabsf(pl) + mi)) {
-          const E x0 = shfl_i(s, 0), x1 = shfl_i(s, 1), x2 = shfl_i(s, 2), x3 = shfl_i(s, 3), x4 = shfl_i(s, 4);
-          exists = less(x1 * x1 + x2 * x2 + x3 * x3, x0 * x4);
+        if (pfp && !(mag > 1e-25f && mag < 1e25f && fabsf(pl - mi) > 1e-5f * mag)) {
+          const double sd = tod(s);
+          const double x0 = shfl_i(sd, 0), x1 = shfl_i(sd, 1), x2 = shfl_i(sd, 2), x3 = shfl_i(sd, 3), x4 = shfl_i(sd, 4);
+          exists = x0 > 0.0 && x0 * x4 > x1 * x1 + x2 * x2 + x3 * x3;
         }
         if (relax && !exists) exists = relax_target<E>(mw, s, lane);
         used = false;
@@ -1271,7 +1301,7 @@ __global__ void __launch_bounds__(256) k_probe_scan(int N, double dv, int mode, 
 #pragma unroll 1
     for (int r = 0; r < reps; r++) {
       cur ^= 1;
-      eval_row<E, false>(sm, N, th, wid, lane, cur, zero);
+      eval_row<E, false>(sm, N, th, wid, lane, cur, zero, 1.0f);
       eval_bar(kTeam);
       ProductMeasure pm;
       pm.prepare(sm.rowsf[cur][0], sm.rowsf[cur][1], sm.rowsf[cur][2]);
