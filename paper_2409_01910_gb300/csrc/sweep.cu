@@ -554,12 +554,21 @@ __device__ __noinline__ bool relax_target(E mw, E& s, int lane) {
   return false;
 }
 
+// One run of a field. WIDE: the fields start on 16 bytes. A field on 8 (a view into a larger array)
+// is read and written by single values, in a kernel of its own: a test of the addresses in the
+// kernel took 2 % of the scan of 64 cells of 32^3.
+template <bool WIDE>
 __device__ __forceinline__ void load_run(const double* p, double (&x)[R]) {
+  if (WIDE) {
 #pragma unroll
-  for (int t = 0; t < R; t += 2) {
-    const double2 v = *reinterpret_cast<const double2*>(p + t);
-    x[t] = v.x;
-    x[t + 1] = v.y;
+    for (int t = 0; t < R; t += 2) {
+      const double2 v = *reinterpret_cast<const double2*>(p + t);
+      x[t] = v.x;
+      x[t + 1] = v.y;
+    }
+  } else {
+#pragma unroll
+    for (int t = 0; t < R; t++) x[t] = p[t];
   }
 }
 
@@ -601,7 +610,7 @@ __device__ __forceinline__ void scan_tables(SweepSmem<E>& sm, const InstDev& I, 
 // The visit of one cell by one cluster. rbuf: this CTA's r (its runs, thread-private slots);
 // den2 (2-D): 1 / (|v1|/dx + |v2|/dy + nu/eps) at [i2][i1].
 // ---------------------------------------------------------------------------------------
-template <typename E, bool TWO_D>
+template <typename E, bool TWO_D, bool WIDE>
 __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I, SweepSmem<E>& sm, E* rbuf, E* den2,
                                            const CellIO& io, cg::cluster_group& cl, int CS, int rank, int& buf,
                                            Tally& ty) {
@@ -673,7 +682,7 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
       const int sgn1 = i1 + 1 - N / 2, sgn2 = i2 + 1 - N / 2;  // v1, v2 in units of dv
       const M v1 = node_m<M, TWO_D>(sm.vm, i1, N), v2 = node_m<M, TWO_D>(sm.vm, i2, N);
       double x[R];
-      load_run(io.f + e0, x);
+      load_run<WIDE>(io.f + e0, x);
       if (pass == 0) {
         E p0 = zero;
 #pragma unroll
@@ -701,16 +710,16 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
       {
         // r = -(|v1|/dx) f_up,x - (|v2|/dy) f_up,y - P/eps - b (upwind neighbours: latest values)
         double pv[R], u1[R], u2[R], bv[R];
-        load_run(io.P + e0, pv);
+        load_run<WIDE>(io.P + e0, pv);
         const int s1 = sgn1 > 0 ? 0 : 1, s2 = sgn2 > 0 ? 2 : 3;
         const double* up1 = sgn1 > 0 ? io.nb[0] : io.nb[1];
         const double* up2 = TWO_D ? (sgn2 > 0 ? io.nb[2] : io.nb[3]) : nullptr;
         const bool g1 = sgn1 != 0 && !up1, g2 = TWO_D && sgn2 != 0 && !up2;
-        if (sgn1 != 0 && up1) load_run(up1 + e0, u1);
+        if (sgn1 != 0 && up1) load_run<WIDE>(up1 + e0, u1);
         if constexpr (TWO_D) {
-          if (sgn2 != 0 && up2) load_run(up2 + e0, u2);
+          if (sgn2 != 0 && up2) load_run<WIDE>(up2 + e0, u2);
         }
-        if (io.b) load_run(io.b + e0, bv);
+        if (io.b) load_run<WIDE>(io.b + e0, bv);
         auto ghost = [&](int side, double(&u)[R]) {
           const E w12 = sm.rho[side] * (sm.W[side][0][i1] * sm.W[side][1][i2]);
 #pragma unroll
@@ -1130,7 +1139,13 @@ __device__ __forceinline__ void visit_cell(const SweepArgs& a, const InstDev& I,
       for (int t = 0; t < R; t += 2) {
         const E x0 = (A * (e12 * sm.ef[2][i30 + t]) - rbuf[slot + t * blockDim.x]) * dn;
         const E x1 = (A * (e12 * sm.ef[2][i30 + t + 1]) - rbuf[slot + (t + 1) * blockDim.x]) * dn;
-        *reinterpret_cast<double2*>(o + t) = make_double2(to_store(x0), to_store(x1));
+        const double d0 = to_store(x0), d1 = to_store(x1);
+        if (WIDE) {
+          *reinterpret_cast<double2*>(o + t) = make_double2(d0, d1);
+        } else {
+          o[t] = d0;
+          o[t + 1] = d1;
+        }
       }
     }
   }
@@ -1150,7 +1165,7 @@ __device__ __forceinline__ void post_tally(const SweepArgs& a, int q, const Tall
   if (threadIdx.x == 0 && ty.status) atomicOr(&a.cnt[q].status, ty.status);
 }
 
-template <typename E>
+template <typename E, bool WIDE>
 __global__ void __launch_bounds__(256) k_sweep(SweepArgs a) {
   cg::cluster_group cl = cg::this_cluster();
   const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
@@ -1182,7 +1197,7 @@ __global__ void __launch_bounds__(256) k_sweep(SweepArgs a) {
     io.nb[2] = io.nb[3] = nullptr;
     io.nu = a.nu[I.cell0 + j];
     io.theta = a.theta + 5 * (long long)(I.cell0 + j);
-    visit_cell<E, false>(a, I, sm, rbuf, nullptr, io, cl, CS, rank, buf, ty);
+    visit_cell<E, false, WIDE>(a, I, sm, rbuf, nullptr, io, cl, CS, rank, buf, ty);
   }
   // no CTA leaves while another may still write its shared memory
   cl.sync();
@@ -1200,7 +1215,7 @@ __global__ void __launch_bounds__(256) k_sweep(SweepArgs a) {
 // Ordering o: 0 SW->NE, 1 NE->SW, 2 NW->SE, 3 SE->NW; wavefront index wf counts from the
 // ordering's starting corner.
 // ---------------------------------------------------------------------------------------
-template <typename E>
+template <typename E, bool WIDE>
 __global__ void __launch_bounds__(256) k_sweep2d(SweepArgs a, int ordering, int wf) {
   cg::cluster_group cl = cg::this_cluster();
   const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
@@ -1237,7 +1252,7 @@ __global__ void __launch_bounds__(256) k_sweep2d(SweepArgs a, int ordering, int 
   io.nb[3] = cj < ny - 1 ? io.f + nx * K : nullptr;
   io.nu = a.nu[I.cell0 + cell];
   io.theta = a.theta + 5 * (long long)(I.cell0 + cell);
-  visit_cell<E, true>(a, I, sm, rbuf, den2, io, cl, CS, rank, buf, ty);
+  visit_cell<E, true, WIDE>(a, I, sm, rbuf, den2, io, cl, CS, rank, buf, ty);
   cl.sync();  // no CTA leaves while another may still write its shared memory
   post_tally(a, 0, ty, 1ULL, rank == 0 && threadIdx.x == 0);
 }
@@ -1341,6 +1356,20 @@ struct ClusterLaunch {
 
 constexpr int kMaxDyn = 160 * 1024;  // dynamic shared memory a scan kernel may be launched with
 
+// The scan kernel of a launch, by arithmetic and by the alignment of its fields.
+bool wide_fields(const SweepArgs& a) {
+  return ((reinterpret_cast<uintptr_t>(a.f) | reinterpret_cast<uintptr_t>(a.P) | reinterpret_cast<uintptr_t>(a.rhs)) &
+          15) == 0;
+}
+const void* sweep_kernel(int arith, bool wide) {
+  if (arith == kSweepDF64) return wide ? (const void*)k_sweep<dfloat, true> : (const void*)k_sweep<dfloat, false>;
+  return wide ? (const void*)k_sweep<double, true> : (const void*)k_sweep<double, false>;
+}
+const void* sweep2d_kernel(int arith, bool wide) {
+  if (arith == kSweepDF64) return wide ? (const void*)k_sweep2d<dfloat, true> : (const void*)k_sweep2d<dfloat, false>;
+  return wide ? (const void*)k_sweep2d<double, true> : (const void*)k_sweep2d<double, false>;
+}
+
 cudaError_t scan_attrs(const void* fn) {
   cudaError_t e = func_attr(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess) e = func_attr(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn);
@@ -1403,7 +1432,7 @@ cudaError_t launch_sweep2d(const SweepArgs& a, const SweepShape& sh, int arith, 
   int cs = sh.cluster;
   while (cs > 1 && ncells * cs > sms) cs /= 2;
   while (cs < 16 && scan_smem(a.N, cs, sh.tpb, true) > 80 * 1024) cs *= 2;
-  const void* fn = arith == kSweepDF64 ? (const void*)k_sweep2d<dfloat> : (const void*)k_sweep2d<double>;
+  const void* fn = sweep2d_kernel(arith, wide_fields(a));
   e = scan_attrs(fn);
   if (e != cudaSuccess) return e;
   ClusterLaunch l(ncells * cs, sh.tpb, cs, scan_smem(a.N, cs, sh.tpb, true), st);
@@ -1419,7 +1448,7 @@ bool sweep_ept_compiled(int ept) {
 
 cudaError_t sweep_max_clusters(int N, const SweepShape& sh, int arith, int* n) {
   *n = 0;
-  const void* fn = arith == kSweepDF64 ? (const void*)k_sweep<dfloat> : (const void*)k_sweep<double>;
+  const void* fn = sweep_kernel(arith, true);
   cudaError_t e = scan_attrs(fn);
   if (e != cudaSuccess) return e;
   ClusterLaunch l(sh.cluster, sh.tpb, sh.cluster, scan_smem(N, sh.cluster, sh.tpb, false), nullptr);
@@ -1437,7 +1466,7 @@ bool sweep_shape_valid(int N, const SweepShape& sh) {
 
 cudaError_t launch_sweep(const SweepArgs& a, const SweepShape& sh, int arith, cudaStream_t st) {
   if (!sweep_shape_valid(a.N, sh)) return cudaErrorInvalidConfiguration;
-  const void* fn = arith == kSweepDF64 ? (const void*)k_sweep<dfloat> : (const void*)k_sweep<double>;
+  const void* fn = sweep_kernel(arith, wide_fields(a));
   cudaError_t e = scan_attrs(fn);
   if (e != cudaSuccess) return e;
   ClusterLaunch l(a.n_inst * sh.cluster, sh.tpb, sh.cluster, scan_smem(a.N, sh.cluster, sh.tpb, false), st);
