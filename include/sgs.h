@@ -310,8 +310,12 @@ int sgs_read_active(sgs_handle* h, int* active, void* stream);
 /* Launch shape of the persistent scan: nodes per thread (ept, a divisor of nv with a
  * compiled kernel: 2, 4, 8, 12, ..., 32), CTAs per cluster (a power of two <= 16; one
  * cluster walks one instance) and threads per CTA (a multiple of 32 in [160, 256]) with
- * ept * cluster * threads >= nv^3. sgs_set_sweep_shape returns SGS_ERR_ARG for an invalid
- * shape and SGS_ERR_UNSUPPORTED for one that cannot be resident on the device. */
+ * ept * cluster * threads >= nv^3. The scans take the cluster and the threads from it (their
+ * threads walk as many nodes as there are); the one inside sgs_dc_step on a 1-D handle holds
+ * ept nodes in each thread. sgs_set_sweep_shape sets the shape of both and returns
+ * SGS_ERR_ARG for an invalid shape and SGS_ERR_UNSUPPORTED for one that cannot be resident
+ * on the device; sgs_autotune may give the scan inside sgs_dc_step one of its own, which
+ * sgs_get_sweep_shape does not show. */
 int sgs_get_sweep_shape(const sgs_handle* h, int* ept, int* cluster, int* threads);
 int sgs_set_sweep_shape(sgs_handle* h, int ept, int cluster, int threads);
 
@@ -327,7 +331,10 @@ typedef struct {
 
 /* Autotuner. Times every valid scan shape on the bound instances (reps forward + backward
  * scan pairs each, after one untimed pair, CUDA events on the stream), keeps the fastest
- * for all later scans and reports it. The timed scans are real SGS scans: f advances by
+ * for all later scans and reports it; shapes that differ in ept only are one candidate. Where
+ * sgs_dc_step has a scan of its own (1-D SGS_FP32 handles), times every shape, ept included,
+ * for that one as well and keeps its fastest for it; the reported ept is the fastest
+ * there for the reported cluster and threads. The timed scans are real SGS scans: f advances by
  * (reps + 1) symmetric sweeps with the given P per candidate. Then times the spectral sum
  * (the handle's arithmetic, all cells, two launches after one untimed one) for every
  * decomposition of 1, 2 or 4 lane groups per block and about 1500, 3000 or 6000 blocks, and

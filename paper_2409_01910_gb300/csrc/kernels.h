@@ -237,6 +237,7 @@ cudaError_t launch_sweep2d(const SweepArgs& a, const SweepShape& sh, int arith, 
 cudaError_t launch_sweep(const SweepArgs& a, const SweepShape& sh, int arith, cudaStream_t st);
 // The double-float scan of sgs_dc_step (sweep_nodes.cu).
 cudaError_t launch_sweep_nodes(const SweepArgs& a, const SweepShape& sh, cudaStream_t st);
+cudaError_t sweep_nodes_max_clusters(const SweepShape& sh, int* n);
 // Fast (Carleman-form) spectral operator on the tensor cores (fast.cu): one chunk of S slots
 // (half-sphere nodes, the loss slot last) for every cell.
 struct FastArgs {

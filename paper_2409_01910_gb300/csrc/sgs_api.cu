@@ -133,7 +133,8 @@ struct sgs_handle {
     std::vector<int> hcell_inst;
   };
   std::vector<Level> lev;
-  SweepShape sweep{8, 1, 256};
+  SweepShape sweep{8, 1, 256};     // of the scans (whose kernels take the cluster and the threads from it)
+  SweepShape sweep_dc{8, 1, 256};  // of the scan inside sgs_dc_step (sweep_nodes.cu)
   int sweep_arith = kSweepF64;
   // profiling: per-class CUDA-event pairs recorded on the launching stream
   bool prof = false;
@@ -812,7 +813,7 @@ int sweep_impl(sgs_handle* h, double* f, const double* P, const double* rhs, int
     if (e != cudaSuccess) return cuda_status(e);
     a.rhs = b2;
   }
-  return cuda_status(h->dc_scan ? launch_sweep_nodes(a, h->sweep, st)
+  return cuda_status(h->dc_scan ? launch_sweep_nodes(a, h->sweep_dc, st)
                                 : launch_sweep(a, h->sweep, h->sweep_arith, st));
 }
 
@@ -1075,6 +1076,17 @@ int time_sum(sgs_handle* h, int reps, cudaStream_t st, float* ms) {
 }
 
 // Times `reps` forward + backward scans of the current launch shape (CUDA events on st).
+// Whether sgs_dc_step of this handle scans with the node-wise kernel.
+bool has_dc_scan(const sgs_handle* h) { return h->precision == SGS_FP32 && h->spectral && !h->two_d; }
+
+// Whether the shape can be resident: as a scan, or (dc) as the scan inside sgs_dc_step.
+bool shape_runs(const sgs_handle* h, const SweepShape& sh, bool dc) {
+  int n = 0;
+  const cudaError_t e = dc ? sweep_nodes_max_clusters(sh, &n) : sweep_max_clusters(h->N, sh, h->sweep_arith, &n);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess && n >= 1;
+}
+
 int time_sweeps(sgs_handle* h, double* f, const double* P, int reps, cudaStream_t st, float* ms) {
   cudaEvent_t a, b;
   if (cudaEventCreate(&a) != cudaSuccess) return SGS_ERR_CUDA;
@@ -1192,7 +1204,7 @@ int sgs_setup(const sgs_problem* problems, int n_inst, sgs_handle** out, size_t*
   }
   layout(h);
   h->sweep_arith = h->precision == SGS_FP32 ? kSweepDF64 : kSweepF64;
-  h->sweep = sweep_shape(h->N, h->sweep_arith);
+  h->sweep = h->sweep_dc = sweep_shape(h->N, h->sweep_arith);
   *out = h;
   if (workspace_bytes) *workspace_bytes = h->ws_bytes;
   return SGS_OK;
@@ -1467,14 +1479,8 @@ int sgs_set_sweep_shape(sgs_handle* h, int ept, int cluster, int threads) {
   if (!h) return SGS_ERR_ARG;
   SweepShape sh{ept, cluster, threads};
   if (!sweep_ept_compiled(ept) || !sweep_shape_valid(h->N, sh)) return SGS_ERR_ARG;
-  int n = 0;
-  cudaError_t e = sweep_max_clusters(h->N, sh, h->sweep_arith, &n);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return SGS_ERR_UNSUPPORTED;
-  }
-  if (n < 1) return SGS_ERR_UNSUPPORTED;
-  h->sweep = sh;
+  if (!shape_runs(h, sh, false) || (has_dc_scan(h) && !shape_runs(h, sh, true))) return SGS_ERR_UNSUPPORTED;
+  h->sweep = h->sweep_dc = sh;
   return SGS_OK;
 }
 
@@ -1484,41 +1490,75 @@ int sgs_autotune(sgs_handle* h, double* f, const double* P, int reps, sgs_tuning
   cudaStream_t st = as_stream(stream);
   const bool prof = h->prof;
   h->prof = false;
-  const SweepShape start = h->sweep;
+  const SweepShape start = h->sweep, start_dc = h->sweep_dc;
   const int K = h->N * h->N * h->N;
-  SweepShape best = start;
-  float best_ms = -1.0f;
-  int tried = 0, r = SGS_OK;
+  std::vector<SweepShape> shapes;
   const int epts[] = {2, 4, 8, 12, 16, 20, 24, 28, 32};
   for (int ept : epts) {
     if (h->N % ept) continue;
     for (int cs = 1; cs <= 16; cs *= 2) {
       int per = (K + ept * cs - 1) / (ept * cs);
       int tpb = (per + 31) / 32 * 32;
-      if (tpb < 160) tpb = 160;  // warps 0-4 serve the Newton evaluations
+      if (tpb < 160) tpb = 160;
       SweepShape sh{ept, cs, tpb};
       if (!sweep_shape_valid(h->N, sh)) continue;
       if ((long long)(tpb - 32) * cs * ept >= K && tpb > 160) continue;  // a whole warp idle in every CTA
-      int n = 0;
-      if (sweep_max_clusters(h->N, sh, h->sweep_arith, &n) != cudaSuccess) {
-        cudaGetLastError();
-        continue;
+      shapes.push_back(sh);
+    }
+  }
+  // Times one candidate into ms (after a warm-up); negative: it cannot run.
+  int tried = 0, r = SGS_OK;
+  auto time_shape = [&](const SweepShape& sh, bool dc, float* ms) {
+    *ms = -1.0f;
+    if (!shape_runs(h, sh, dc)) return;
+    (dc ? h->sweep_dc : h->sweep) = sh;
+    h->dc_scan = dc;
+    float t = 0.0f;
+    r = time_sweeps(h, f, P, 1, st, &t);
+    if (r == SGS_OK) r = time_sweeps(h, f, P, reps, st, &t);
+    h->dc_scan = false;
+    if (r != SGS_OK) return;
+    tried++;
+    *ms = t;
+  };
+  auto same_launch = [](const SweepShape& a, const SweepShape& b) { return a.cluster == b.cluster && a.tpb == b.tpb; };
+  // The scans take the cluster and the threads only: shapes that differ in the nodes per thread are
+  // one launch.
+  SweepShape best = start;
+  float best_ms = -1.0f;
+  for (size_t i = 0; i < shapes.size() && r == SGS_OK; i++) {
+    bool seen = false;
+    for (size_t k = 0; k < i; k++) seen = seen || same_launch(shapes[k], shapes[i]);
+    if (seen) continue;
+    float ms;
+    time_shape(shapes[i], false, &ms);
+    if (ms >= 0.0f && (best_ms < 0.0f || ms < best_ms)) {
+      best_ms = ms;
+      best = shapes[i];
+    }
+  }
+  // The scan inside sgs_dc_step is another kernel and keeps the shape that suits it. The shape that is
+  // reported has its fastest nodes per thread for that cluster and these threads, so that a
+  // handle that is given it runs a timed one of either kernel.
+  SweepShape best_dc = start_dc;
+  if (has_dc_scan(h)) {
+    float best_dc_ms = -1.0f, best_ept_ms = -1.0f;
+    for (size_t i = 0; i < shapes.size() && r == SGS_OK; i++) {
+      float ms;
+      time_shape(shapes[i], true, &ms);
+      if (ms < 0.0f) continue;
+      if (best_dc_ms < 0.0f || ms < best_dc_ms) {
+        best_dc_ms = ms;
+        best_dc = shapes[i];
       }
-      if (n < 1) continue;
-      h->sweep = sh;
-      float ms = 0.0f;
-      r = time_sweeps(h, f, P, 1, st, &ms);  // warm-up
-      if (r == SGS_OK) r = time_sweeps(h, f, P, reps, st, &ms);
-      if (r != SGS_OK) break;
-      tried++;
-      if (best_ms < 0.0f || ms < best_ms) {
-        best_ms = ms;
-        best = sh;
+      if (same_launch(shapes[i], best) && (best_ept_ms < 0.0f || ms < best_ept_ms)) {
+        best_ept_ms = ms;
+        best.ept = shapes[i].ept;
       }
     }
-    if (r != SGS_OK) break;
   }
   h->sweep = r == SGS_OK ? best : start;
+  h->sweep_dc = r == SGS_OK ? best_dc : start_dc;
   if (r != SGS_OK) {
     h->prof = prof;
     return r;

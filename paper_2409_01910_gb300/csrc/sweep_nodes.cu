@@ -827,40 +827,59 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
   if (tid == 0 && status) atomicOr(&a.cnt[q].status, status);
 }
 
-template <int EPT>
-cudaError_t launch_nodes_t(const SweepArgs& a, const SweepShape& sh, cudaStream_t st) {
-  cudaError_t e = func_attr((const void*)k_sweep_nodes<dfloat, EPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.n_inst * sh.cluster);
-  cfg.blockDim = dim3(sh.tpb);
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = sh.cluster;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_sweep_nodes<dfloat, EPT>, a);
+// The kernel of a shape (null: not compiled) and its launch configuration.
+const void* nodes_kernel(int ept) {
+  switch (ept) {
+    case 2: return (const void*)k_sweep_nodes<dfloat, 2>;
+    case 4: return (const void*)k_sweep_nodes<dfloat, 4>;
+    case 8: return (const void*)k_sweep_nodes<dfloat, 8>;
+    case 12: return (const void*)k_sweep_nodes<dfloat, 12>;
+    case 16: return (const void*)k_sweep_nodes<dfloat, 16>;
+    case 20: return (const void*)k_sweep_nodes<dfloat, 20>;
+    case 24: return (const void*)k_sweep_nodes<dfloat, 24>;
+    case 28: return (const void*)k_sweep_nodes<dfloat, 28>;
+    case 32: return (const void*)k_sweep_nodes<dfloat, 32>;
+  }
+  return nullptr;
 }
+
+struct NodesLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  NodesLaunch(const SweepShape& sh, int n_inst, cudaStream_t st) {
+    cfg.gridDim = dim3(n_inst * sh.cluster);
+    cfg.blockDim = dim3(sh.tpb);
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = sh.cluster;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+};
 
 }  // namespace
 
 cudaError_t launch_sweep_nodes(const SweepArgs& a, const SweepShape& sh, cudaStream_t st) {
-  if (!sweep_shape_valid(a.N, sh)) return cudaErrorInvalidConfiguration;
-  switch (sh.ept) {
-    case 2: return launch_nodes_t<2>(a, sh, st);
-    case 4: return launch_nodes_t<4>(a, sh, st);
-    case 8: return launch_nodes_t<8>(a, sh, st);
-    case 12: return launch_nodes_t<12>(a, sh, st);
-    case 16: return launch_nodes_t<16>(a, sh, st);
-    case 20: return launch_nodes_t<20>(a, sh, st);
-    case 24: return launch_nodes_t<24>(a, sh, st);
-    case 28: return launch_nodes_t<28>(a, sh, st);
-    case 32: return launch_nodes_t<32>(a, sh, st);
-  }
-  return cudaErrorInvalidConfiguration;
+  const void* fn = nodes_kernel(sh.ept);
+  if (!fn || !sweep_shape_valid(a.N, sh)) return cudaErrorInvalidConfiguration;
+  cudaError_t e = func_attr(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  NodesLaunch l(sh, a.n_inst, st);
+  SweepArgs args = a;
+  void* p[] = {&args};
+  return cudaLaunchKernelExC(&l.cfg, fn, p);
+}
+
+cudaError_t sweep_nodes_max_clusters(const SweepShape& sh, int* n) {
+  *n = 0;
+  const void* fn = nodes_kernel(sh.ept);
+  if (!fn) return cudaErrorInvalidConfiguration;
+  cudaError_t e = func_attr(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  NodesLaunch l(sh, 1, nullptr);
+  return cudaOccupancyMaxActiveClusters(n, fn, &l.cfg);
 }
 
 }  // namespace sgs

@@ -58,6 +58,25 @@ def test_fast_along_the_walls_1d(oracle, U):
     assert rel(got, fo) <= tol(U, T)
 
 
+@pytest.mark.parametrize("precision", [sgs.FP64, sgs.FP32])
+@pytest.mark.parametrize("N,L,T,U", [(16, 6.0, 0.3, (3.0, 0.0, 0.0)), (24, 6.0, 0.2, (3.0, 1.5, 0.5)),
+                                     (32, 8.0, 0.25, (5.0, 0.5, 0.5))])
+def test_cold_fast_gas(oracle, N, L, T, U, precision):
+    """Newton's closing step is taken with an FP32 direction from raw moments, whose rounding grows
+    with the speed, as that of an evaluation does."""
+    J = 3
+    kw = dict(eps=0.05, total_mass=1.0, inner_fixed=4, bc_kind=(sgs.INFLOW, sgs.INFLOW), bc_u=(U, U), bc_T=(T, T))
+    op = oracle.Problem(N=N, L=L, J=J, kernel=oracle.BGK, **kw)
+    f0, P0 = state(J, N, L, U, T)
+    got, st = gpu_scan(sgs.Problem(nx=J, nv=N, v_max=L, collision=sgs.BGK, precision=precision, **kw), f0, P0, [0, 1])
+    assert st["status"] == 0 and st["inner_iters"] == 2 * 4 * J, st
+    fo = f0.copy()
+    nu = np.array([oracle.collision_frequency(op, x) for x in f0])
+    for d in (+1, -1):
+        oracle.sweep(op, fo, P0, nu, d)
+    assert rel(got, fo) <= (1.0 if precision == sgs.FP64 else 10.0) * tol(U, T)
+
+
 def test_fast_along_the_walls_2d(oracle):
     N, nx, ny, L, T, U = 32, 2, 1, 8.0, 0.25, (0.1, 0.2, 5.0)
     kw = dict(eps=0.2, total_mass=1.0, inner_tol=1e-9, bc_kind=(sgs.INFLOW, sgs.INFLOW), bc_u=(U, U), bc_T=(T, T))
