@@ -1307,17 +1307,24 @@ static size_t dft_smem(int N, int extra_cplx, int extra_real) {
   return 2 * N * N * sizeof(T) + extra_cplx * sizeof(CT) + extra_real * sizeof(T);
 }
 
+// Lane groups per block of a sum over `groups` of them that takes F steps at once: as many as asked
+// for, within an SM's shared memory.
+static size_t sum_group_bytes(int BK, int elem_bytes) {
+  return (size_t)2 * (2 * (4 * BK - 1) + 1) * kLanes * 2 * elem_bytes;
+}
+static size_t sum_weight_bytes(int BK, int elem_bytes, int F) {
+  return 2 * F * ((size_t)sum_pad(2 * BK - 1, elem_bytes) * elem_bytes + (F > 1 ? 16 : 0));
+}
+static int sum_groups(int BK, int elem_bytes, int F, int NW, int groups) {
+  const int fit = (int)((220 * 1024 - sum_weight_bytes(BK, elem_bytes, F)) / sum_group_bytes(BK, elem_bytes));
+  return std::max(1, std::min(std::min(NW, groups), fit));
+}
+
 template <typename T, int BK, int F>
 static cudaError_t launch_sum_f(const SumArgs<T>& a, int NW, int n_units, cudaStream_t st) {
-  typedef typename CplxOf<T>::type CT;
-  constexpr int n = 4 * BK - 1;
-  constexpr int VEC = 16 / (int)sizeof(T);
-  constexpr int PWS = (sum_weights(BK) + VEC - 1) / VEC * VEC + (F > 1 ? VEC : 0);
-  // lane groups per block: as many as asked for, within an SM's shared memory
-  constexpr size_t wbytes = 2 * F * PWS * sizeof(T), gbytes = (size_t)2 * (2 * n + 1) * kLanes * sizeof(CT);
   const int groups = a.G - a.g0;
-  const int NG = std::max(1, std::min(std::min(NW, groups), (int)((220 * 1024 - wbytes) / gbytes)));
-  const size_t smem = wbytes + NG * gbytes;
+  const int NG = sum_groups(BK, sizeof(T), F, NW, groups);
+  const size_t smem = sum_weight_bytes(BK, sizeof(T), F) + NG * sum_group_bytes(BK, sizeof(T));
   cudaError_t e = func_attr((const void*)k_sum<T, BK, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid(n_units, (groups + NG - 1) / NG);
@@ -1346,6 +1353,16 @@ static cudaError_t launch_sum_t(const SumArgs<T>& a, int NW, int n_units, cudaSt
 int sum_pad(int H, int elem_bytes) {
   int NP = sum_weights((H + 1) / 2), VEC = 16 / elem_bytes;
   return (NP + VEC - 1) / VEC * VEC;
+}
+
+template <typename T>
+SumShape sum_shape(const SumArgs<T>& a, int H, int NW, int n_units) {
+  const int BK = (H + 1) / 2, folded = a.fold > 1 ? 1 : 0, rest = a.G - folded;
+  SumShape x;
+  x.launches = (rest > 0 ? 1 : 0) + folded;
+  x.warps = rest > 0 ? sum_groups(BK, sizeof(T), 1, NW, rest) : 1;
+  x.blocks = n_units * ((rest + x.warps - 1) / x.warps + folded);
+  return x;
 }
 
 template <typename T>
@@ -1501,6 +1518,8 @@ cudaError_t launch_build_weights_lo(const int4* units, const long long* unit_ste
 
 template cudaError_t launch_dft<double>(const double*, const CollideCtx<double>&, const DftMode&, cudaStream_t);
 template cudaError_t launch_dft<float>(const double*, const CollideCtx<float>&, const DftMode&, cudaStream_t);
+template SumShape sum_shape<double>(const SumArgs<double>&, int, int, int);
+template SumShape sum_shape<float>(const SumArgs<float>&, int, int, int);
 template cudaError_t launch_spectral_sum<double>(const CollideCtx<double>&, double2*, cudaStream_t);
 template cudaError_t launch_spectral_sum<float>(const CollideCtx<float>&, float2*, cudaStream_t);
 template cudaError_t launch_reduce_idft<double>(const double*, double*, double*, const CollideCtx<double>&,

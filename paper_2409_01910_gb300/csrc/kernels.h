@@ -202,6 +202,13 @@ cudaError_t launch_collide_bgk(const double* f, const CellTables& ct, int C, int
                                const double* nu, double* Q, double* P, cudaStream_t st);
 template <typename T>
 cudaError_t launch_dft(const double* f, const CollideCtx<T>& x, const DftMode& md, cudaStream_t st);
+// What a spectral sum launches: kernels (a folded last lane group is one of its own), blocks of all of
+// them, and lane groups per block of the unfolded one.
+struct SumShape {
+  int launches, blocks, warps;
+};
+template <typename T>
+SumShape sum_shape(const SumArgs<T>& a, int H, int NW, int n_units);
 template <typename T>
 cudaError_t launch_spectral_sum(const CollideCtx<T>& x, typename CplxOf<T>::type* partial, cudaStream_t st);
 template <typename T>

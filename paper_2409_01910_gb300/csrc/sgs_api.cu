@@ -671,7 +671,8 @@ int collide_impl(sgs_handle* h, const double* f, double* Q, double* P, int preci
     }
     if (er != cudaSuccess) return cuda_status(er);
     {
-      Scope sc(h, precision == SGS_FP64 ? SGS_PROF_SUM_FP64 : SGS_PROF_SUM, st, 1, x.C);
+      Scope sc(h, precision == SGS_FP64 ? SGS_PROF_SUM_FP64 : SGS_PROF_SUM, st,
+               sum_shape(x.sum, x.H, x.NW, x.n_units).launches, x.C);
       er = launch_spectral_sum(x, nullptr, st);
     }
     if (er != cudaSuccess) return cuda_status(er);
@@ -1605,9 +1606,11 @@ int sgs_autotune(sgs_handle* h, double* f, const double* P, int reps, sgs_tuning
     out->sweep_threads = best.tpb;
     out->sweep_ms = best_ms / reps;
     out->candidates = tried;
-    out->sum_warps = h->NW;
+    auto shape = [](const auto& x) { return sum_shape(x.sum, x.H, x.NW, x.n_units); };
+    const SumShape sum = h->precision == SGS_FP32 ? shape(collide_ctx<float>(h)) : shape(collide_ctx<double>(h));
+    out->sum_warps = sum.warps;
     out->sum_units = (int)h->units.size();
-    out->sum_blocks = (int)h->units.size() * ((h->G + h->NW - 1) / h->NW);
+    out->sum_blocks = sum.blocks;
     out->sum_ms = sum_best > 0.0f ? sum_best / 2 : 0.0f;
     out->sum_candidates = sum_tried;
   }
