@@ -509,7 +509,7 @@ def roofline(cls, prof, wl, sm_mhz, peaks, stats=None):
         # doubles; 2-D: 7 K doubles)
         byts = (7 if is_cavity(wl) else 5) * K * 8 * cells
         ach = byts / (ms * 1e-3) / 1e9
-        out = {"kernel": "k_sweep<dfloat,8> (persistent SGS scan, one cluster per instance)", "bound": "hbm",
+        out = {"kernel": "k_sweep<dfloat> (persistent SGS scan, one cluster per instance)", "bound": "hbm",
                "achieved": ach, "peak": hbm["hbm_gbs"], "unit": "GB/s", "frac": ach / hbm["hbm_gbs"],
                "traffic": kernel_traffic("k_sweep<dfloat,8>", cells / max(1, n)),
                "traffic_per": f"launch of {cells / max(1, n):.0f} cell visits",

@@ -1426,7 +1426,8 @@ cudaError_t launch_dft(const double* f, const CollideCtx<T>& x, const DftMode& m
   k_dft_i2<T><<<dim3(C, N), 256, sm2, st>>>(x.sb, N);
   e = func_attr((const void*)k_dft_i1<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
   if (e != cudaSuccess) return e;
-  // groups beyond the last cell keep the zeros written at bind time
+  // lanes beyond the last cell hold anything and are never read back: no lane of a sum reads another
+  // one's cell (a folded group's lanes are those of its cells)
   k_dft_i1<T><<<dim3(C, n), 256, sm2, st>>>(x.sb, N);
   return cudaGetLastError();
 }
@@ -1458,7 +1459,7 @@ cudaError_t launch_reduce_idft(const double* f, double* Q, double* P, const Coll
   size_t sm4 = dft_smem<T>(N, N * n, 0);
   e = func_attr((const void*)k_idft_k3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm4);
   if (e != cudaSuccess) return e;
-  // the factors of this collision step were written by launch_dft
+  // the factors of this collision step were written by launch_moments
   k_idft_k3<T><<<dim3(C, N), 256, sm4, st>>>(x.sb, f, x.ct, x.efac, x.nu, Q, P, N, x.dv, Qadd, x.mom);
   e = cudaGetLastError();
   if (e != cudaSuccess || !x.mom) return e;

@@ -232,7 +232,7 @@ struct SweepShape {
 // arithmetic of the sweep's elementwise work and reductions
 constexpr int kSweepF64 = 0;   // native FP64
 constexpr int kSweepDF64 = 1;  // double-float on the FP32 pipes (FP64-class accuracy)
-SweepShape sweep_shape(int N, int arith);
+SweepShape sweep_shape(int N);
 bool sweep_shape_valid(int N, const SweepShape& sh);
 // Sweep launch shapes: nodes per thread with a compiled kernel, and the number of clusters of
 // the shape that fit on the device at once (0: the shape cannot run).

@@ -1076,7 +1076,6 @@ int time_sum(sgs_handle* h, int reps, cudaStream_t st, float* ms) {
   return cuda_status(e);
 }
 
-// Times `reps` forward + backward scans of the current launch shape (CUDA events on st).
 // Whether sgs_dc_step of this handle scans with the node-wise kernel.
 bool has_dc_scan(const sgs_handle* h) { return h->precision == SGS_FP32 && h->spectral && !h->two_d; }
 
@@ -1088,6 +1087,7 @@ bool shape_runs(const sgs_handle* h, const SweepShape& sh, bool dc) {
   return e == cudaSuccess && n >= 1;
 }
 
+// Times `reps` forward + backward scans of the current launch shape (CUDA events on st).
 int time_sweeps(sgs_handle* h, double* f, const double* P, int reps, cudaStream_t st, float* ms) {
   cudaEvent_t a, b;
   if (cudaEventCreate(&a) != cudaSuccess) return SGS_ERR_CUDA;
@@ -1205,7 +1205,7 @@ int sgs_setup(const sgs_problem* problems, int n_inst, sgs_handle** out, size_t*
   }
   layout(h);
   h->sweep_arith = h->precision == SGS_FP32 ? kSweepDF64 : kSweepF64;
-  h->sweep = h->sweep_dc = sweep_shape(h->N, h->sweep_arith);
+  h->sweep = h->sweep_dc = sweep_shape(h->N);
   *out = h;
   if (workspace_bytes) *workspace_bytes = h->ws_bytes;
   return SGS_OK;

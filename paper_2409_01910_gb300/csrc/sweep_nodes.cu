@@ -35,7 +35,8 @@ namespace {
 
 constexpr int kRedMax = 10;  // values per cluster reduction
 
-template <typename E>
+typedef dfloat E;  // the arithmetic of the sums and the elementwise work
+
 struct NodesSmem {
   E vv[kMaxN];         // nodes v_i
   E vq[kMaxN];         // v_i^2
@@ -50,11 +51,11 @@ struct NodesSmem {
   E Sb[2][4][5];       // Newton evaluations, double-buffered: row r = sums of evaluating warp r
   E Gs[3][6];          // per-dimension sums for the norm of M+ - M[g] (derived residual)
   E svE[5];            // step-1 target s
-  E W3[4][kMaxN];      // third factor of each wall's unit Maxwellian
+  E W3[2][kMaxN];      // third factor of each wall's unit Maxwellian
   E red_warp[32][kRedMax];
   E red_tote[kRedMax];
   E thE[5];            // trial theta in E
-  E scal[6];           // per-visit scalars: wall densities of the sides, nu/eps
+  E scal[3];           // per-visit scalars: wall densities of the sides, nu/eps
   double red_part[2][kRedMax];
   double red_tot[kRedMax];
   double thg[5], thp[5];
@@ -69,7 +70,7 @@ __device__ __forceinline__ dfloat shfl_i(dfloat v, int lane) { return {shfl_i(v.
 // additions are those of a butterfly over all values (warp_allsum: the same pairs at every level,
 // and an addition is commutative), but in each of the first three steps a lane keeps half of its
 // values and hands over the other half, so there are 9 of them instead of 5 NV.
-template <int NV, typename E>
+template <int NV>
 __device__ __forceinline__ E warp_sums(const E (&x)[NV], int lane) {
   E v[8];
 #pragma unroll
@@ -108,11 +109,11 @@ __device__ __forceinline__ int clearly_exists(float f0, float f1, float f2, floa
 // Cluster-wide sum of NV values per thread; tot (double) and sm.red_tote (E) receive the
 // totals, identical in every CTA.
 // ---------------------------------------------------------------------------------------
-template <int NV, typename E>
-__device__ inline void cluster_reduce(E (&v)[NV], double (&tot)[NV], NodesSmem<E>& sm, int& buf,
+template <int NV>
+__device__ inline void cluster_reduce(E (&v)[NV], double (&tot)[NV], NodesSmem& sm, int& buf,
                                       cg::cluster_group& cl, int CS) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const E ws = warp_sums<NV, E>(v, lane);
+  const E ws = warp_sums<NV>(v, lane);
   if ((lane & 3) == 0 && (lane >> 2) < NV) sm.red_warp[wid][lane >> 2] = ws;
   __syncthreads();
   if (threadIdx.x < NV) {
@@ -147,8 +148,7 @@ __device__ inline void cluster_reduce(E (&v)[NV], double (&tot)[NV], NodesSmem<E
 // Newton for the discrete Maxwellian, executed by the whole CTA with uniform control flow.
 // ---------------------------------------------------------------------------------------
 // Warps 0-2: factors and 1-D sums S_d^p of dimension d at the trial theta in sm.thE.
-template <typename E>
-__device__ __noinline__ void eval_cta(NodesSmem<E>& sm, int N) {
+__device__ __noinline__ void eval_cta(NodesSmem& sm, int N) {
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (wid < 4) {
     // warps 0-2: dimension d; warp 3: dimension 1 again, weighted by |v1|/dx (step 1, eq. (24))
@@ -167,14 +167,13 @@ __device__ __noinline__ void eval_cta(NodesSmem<E>& sm, int N) {
     s[2] = e * sm.vq[lane];
     s[3] = s[2] * sm.vv[lane];
     s[4] = s[2] * sm.vq[lane];
-    const E t = warp_sums<5, E>(s, lane);
+    const E t = warp_sums<5>(s, lane);
     if ((lane & 3) == 0 && lane < 20) (wid < 3 ? sm.S[d] : sm.S1w)[lane >> 2] = t;
   }
   __syncthreads();
 }
 
 // Moments (E) and Jacobian (FP32) of the separable Maxwellian from its three 1-D sums.
-template <typename E>
 __device__ inline void moments_from_sums(const E* S1, const E* S2, const E* S3, E (&mom)[5], float (&Aa)[15]) {
   E s23 = S2[0] * S3[0];
   mom[0] = S1[0] * s23;
@@ -203,9 +202,9 @@ __device__ inline void moments_from_sums(const E* S1, const E* S2, const E* S3, 
 }
 
 // Component k of a five-element register array (static indices only).
-template <typename E>
-__device__ inline E pick5(const E (&v)[5], int k) {
-  E r = v[0];
+template <typename T>
+__device__ inline T pick5(const T (&v)[5], int k) {
+  T r = v[0];
 #pragma unroll
   for (int q = 1; q < 5; q++)
     if (k == q) r = v[q];
@@ -214,7 +213,6 @@ __device__ inline E pick5(const E (&v)[5], int k) {
 
 // Lane k < 5 returns moment k, with the operations of moments_from_sums (lanes 5 and 6 form parts of
 // the last one), so that a warp does a handful of double-float operations instead of forty.
-template <typename E>
 __device__ __forceinline__ E lane_moment(const E* S1, const E* S2, const E* S3, int lane) {
   const int i = lane == 1 ? 1 : (lane == 4 ? 2 : 0), j = lane == 2 ? 1 : (lane == 5 ? 2 : 0),
             l = lane == 3 ? 1 : (lane == 6 ? 2 : 0);
@@ -229,10 +227,9 @@ __device__ __forceinline__ E lane_moment(const E* S1, const E* S2, const E* S3, 
 
 // Residual of the moments against the target (lane k: component k of it, tl), in Ff on every
 // lane, the Jacobian (FP32) and the scaled residual norm, from the 1-D sums. it0: |target_0|.
-template <typename E>
 __device__ __forceinline__ void combine(const E* S1, const E* S2, const E* S3, E w, E tl, float it0, float (&Ff)[5],
                                         float (&A)[15], float& fn) {
-  const float Fl = tof(w * lane_moment<E>(S1, S2, S3, threadIdx.x & 31) - tl);
+  const float Fl = tof(w * lane_moment(S1, S2, S3, threadIdx.x & 31) - tl);
   float amax = 0.0f;
 #pragma unroll
   for (int i = 0; i < 5; i++) {
@@ -242,7 +239,7 @@ __device__ __forceinline__ void combine(const E* S1, const E* S2, const E* S3, E
   fn = amax / it0;
   E mom[5];
   float Aa[15];
-  moments_from_sums<E>(S1, S2, S3, mom, Aa);
+  moments_from_sums(S1, S2, S3, mom, Aa);
   const float cf = tof(w);
 #pragma unroll
   for (int i = 0; i < 15; i++) A[i] = cf * Aa[i];
@@ -252,8 +249,7 @@ __device__ __forceinline__ void combine(const E* S1, const E* S2, const E* S3, E
 // dimension 1 weighted by |v1|/dx) at the trial theta, of which lane k holds component k: factors
 // of warps 0-2 to sm.ef, the five 1-D sums to row wid of sm.Sb[buf]. The same arithmetic as
 // eval_cta.
-template <typename E>
-__device__ __forceinline__ void eval_warp(NodesSmem<E>& sm, int N, E thl, int wid, int buf) {
+__device__ __forceinline__ void eval_warp(NodesSmem& sm, int N, E thl, int wid, int buf) {
   const int lane = threadIdx.x & 31;
   const int d = wid == 3 ? 0 : wid;
   const E b = shfl_i(thl, 1 + d), g = shfl_i(thl, 4), al = shfl_i(thl, 0);
@@ -271,7 +267,7 @@ __device__ __forceinline__ void eval_warp(NodesSmem<E>& sm, int N, E thl, int wi
   s[2] = e * sm.vq[lane];
   s[3] = s[2] * sm.vv[lane];
   s[4] = s[2] * sm.vq[lane];
-  const E t = warp_sums<5, E>(s, lane);
+  const E t = warp_sums<5>(s, lane);
   if ((lane & 3) == 0 && lane < 20) sm.Sb[buf][wid][lane >> 2] = t;
 }
 
@@ -294,8 +290,7 @@ __device__ __forceinline__ void eval_bar(int nwarps) {
 // and thread-0 broadcasts of a split design. The FP64 theta is spread over the lanes (lane k:
 // component k), the moments and sums too, so an iteration takes one FP64 instruction. With every
 // component on lane 0 it took five of them and six conversions, about half of its 1.5 us.
-template <typename E>
-__device__ __noinline__ int newton_cta(NodesSmem<E>& sm, int N, E w, bool weighted, const E* target, double* th,
+__device__ __noinline__ int newton_cta(NodesSmem& sm, int N, E w, bool weighted, const E* target, double* th,
                                        double L, double tol, int maxit, bool have_eval) {
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int nev = 4;
@@ -307,16 +302,16 @@ __device__ __noinline__ int newton_cta(NodesSmem<E>& sm, int N, E w, bool weight
   if (wid < nev) {
     const int kl = min(lane, 4);  // this lane's component
     double thl = th[kl];
-    const E tl = pick5<E>(*reinterpret_cast<const E(*)[5]>(target), kl);
+    const E tl = pick5(*reinterpret_cast<const E(*)[5]>(target), kl);
     const float it0 = fabsf(tof(target[0]));
     float Ff[5], A[15], fn = 0.0f;
     int buf = 0, last = -1;  // last: buffer of the latest evaluation (-1: the canonical sums)
     if (have_eval) {
-      combine<E>(weighted ? sm.S1w : sm.S[0], sm.S[1], sm.S[2], w, tl, it0, Ff, A, fn);
+      combine(weighted ? sm.S1w : sm.S[0], sm.S[1], sm.S[2], w, tl, it0, Ff, A, fn);
     } else {
-      eval_warp<E>(sm, N, cvt<E>(thl), wid, buf);
+      eval_warp(sm, N, cvt<E>(thl), wid, buf);
       eval_bar(nev);
-      combine<E>(sm.Sb[buf][weighted ? 3 : 0], sm.Sb[buf][1], sm.Sb[buf][2], w, tl, it0, Ff, A, fn);
+      combine(sm.Sb[buf][weighted ? 3 : 0], sm.Sb[buf][1], sm.Sb[buf][2], w, tl, it0, Ff, A, fn);
       last = buf;
       buf ^= 1;
     }
@@ -331,15 +326,15 @@ __device__ __noinline__ int newton_cta(NodesSmem<E>& sm, int N, E w, bool weight
         const float Lf = (float)L;
         const float stepf = fabsf(y[0]) + Lf * (fabsf(y[1]) + fabsf(y[2]) + fabsf(y[3])) + Lf * Lf * fabsf(y[4]);
         // -D A^{-1} F, D = diag(1,1,1,1,-1)
-        const float yl = pick5<float>(y, kl);
+        const float yl = pick5(y, kl);
         const double dirl = widen(kl == 4 ? yl : -yl);
         float lam = 1.0f;
         double lamd = 1.0, tt;
         for (int hv = 0; hv < 40; hv++) {
           tt = fma(lamd, dirl, thl);
-          eval_warp<E>(sm, N, cvt<E>(tt), wid, buf);
+          eval_warp(sm, N, cvt<E>(tt), wid, buf);
           eval_bar(nev);
-          combine<E>(sm.Sb[buf][weighted ? 3 : 0], sm.Sb[buf][1], sm.Sb[buf][2], w, tl, it0, Ff, A, fn);
+          combine(sm.Sb[buf][weighted ? 3 : 0], sm.Sb[buf][1], sm.Sb[buf][2], w, tl, it0, Ff, A, fn);
           last = buf;
           buf ^= 1;
           if (fn == fn && (fn <= fn_cur || fn <= 1e-10f)) {
@@ -371,8 +366,7 @@ __device__ __noinline__ int newton_cta(NodesSmem<E>& sm, int N, E w, bool weight
   return sm.nret;
 }
 
-template <typename E>
-__device__ inline void copy_factors(NodesSmem<E>& sm, E (*dst)[kMaxN]) {
+__device__ inline void copy_factors(NodesSmem& sm, E (*dst)[kMaxN]) {
   if (threadIdx.x < 3 * kMaxN) {
     int d = threadIdx.x / kMaxN, i = threadIdx.x % kMaxN;
     dst[d][i] = sm.ef[d][i];
@@ -380,25 +374,19 @@ __device__ inline void copy_factors(NodesSmem<E>& sm, E (*dst)[kMaxN]) {
   __syncthreads();
 }
 
-// M[g] of the moments in mom: warm start from th0 (if any; have_eval: the last evaluation is
-// at th0), then from the continuum Maxwellian; on failure keeps th0 (status reported).
+// M[g] of the moments in mom: warm start from th0 (have_eval: the last evaluation is at th0),
+// then from the continuum Maxwellian; on failure keeps th0 (status reported).
 // Result in sm.thg and sm.Eg; the last evaluation is at sm.thg afterwards.
-template <typename E>
-__device__ __noinline__ int solve_mg(NodesSmem<E>& sm, int N, E w, const E* mom, const double* th0, bool have_eval,
+__device__ __noinline__ int solve_mg(NodesSmem& sm, int N, E w, const E* mom, const double* th0, bool have_eval,
                                      double L, double tol, int maxit, unsigned& status) {
   const int tid = threadIdx.x;
   double keep[5];
-  if (th0) {
 #pragma unroll
-    for (int k = 0; k < 5; k++) keep[k] = th0[k];
-  }
+  for (int k = 0; k < 5; k++) keep[k] = th0[k];
   __syncthreads();
-  int it = -1;
-  if (th0) {
-    if (tid < 5) sm.thg[tid] = keep[tid];
-    __syncthreads();
-    it = newton_cta<E>(sm, N, w, false, mom, sm.thg, L, tol, maxit, have_eval);
-  }
+  if (tid < 5) sm.thg[tid] = keep[tid];
+  __syncthreads();
+  int it = newton_cta(sm, N, w, false, mom, sm.thg, L, tol, maxit, have_eval);
   if (it < 0) {
     if (tid == 0) {
       double tg[5];
@@ -409,24 +397,20 @@ __device__ __noinline__ int solve_mg(NodesSmem<E>& sm, int N, E w, const E* mom,
     }
     __syncthreads();
     if (sm.ctl) {
-      it = newton_cta<E>(sm, N, w, false, mom, sm.thg, L, tol, maxit, false);
+      it = newton_cta(sm, N, w, false, mom, sm.thg, L, tol, maxit, false);
     } else {
       status |= SGS_ST_NONPOSITIVE;
     }
   }
   if (it < 0) {
     status |= SGS_ST_NEWTON_FAIL;
-    if (th0 && tid < 5) sm.thg[tid] = keep[tid];
-    // no warm start and no admissible guess (non-positive moments): a fixed theta (the unit
-    // Maxwellian's), so that every CTA of the cluster continues from the same data and takes
-    // the same decisions
-    if (!th0 && !sm.ctl && tid < 5) sm.thg[tid] = tid == 0 ? -1.5 * log(2.0 * kPi) : (tid == 4 ? 0.5 : 0.0);
+    if (tid < 5) sm.thg[tid] = keep[tid];
     __syncthreads();
     if (tid < 5) sm.thE[tid] = cvt<E>(sm.thg[tid]);
     __syncthreads();
-    eval_cta<E>(sm, N);
+    eval_cta(sm, N);
   }
-  copy_factors<E>(sm, sm.Eg);
+  copy_factors(sm, sm.Eg);
   return it;
 }
 
@@ -436,11 +420,10 @@ __device__ __noinline__ int solve_mg(NodesSmem<E>& sm, int N, E w, const E* mom,
 // step-1 weight; its moments come from the separable sums of the last evaluation, which is
 // M[g]'s). 1 + tau = 2, 4, 8, ...: the first target that passes eq. (26) replaces sd and
 // sm.svE. Returns whether one was found.
-template <typename E>
-__device__ inline bool relax_target(NodesSmem<E>& sm, E w, double (&sd)[5]) {
+__device__ inline bool relax_target(NodesSmem& sm, E w, double (&sd)[5]) {
   E m1[5];
   float Aa[15];
-  moments_from_sums<E>(sm.S1w, sm.S[1], sm.S[2], m1, Aa);
+  moments_from_sums(sm.S1w, sm.S[1], sm.S[2], m1, Aa);
   double mw[5];
 #pragma unroll
   for (int k = 0; k < 5; k++) mw[k] = tod(w * m1[k]);
@@ -471,20 +454,18 @@ __device__ inline bool relax_target(NodesSmem<E>& sm, E w, double (&sd)[5]) {
 // from the separable sums of the last evaluation (M[g]'s), the moments of M+ and those of
 // g. No pass over the nodes and no cluster reduction. Warps 0-2 form the sums; the caller's
 // thread 0 takes the decisions. Returns the squared norm sum_k (M+ - M[g])^2 in thread 0.
-template <typename E>
-__device__ inline void derived_sums(NodesSmem<E>& sm) {
+__device__ inline void derived_sums(NodesSmem& sm) {
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (wid < 3) {
     const E p = sm.Ep[wid][lane], q = sm.Eg[wid][lane], dl = q - p;
     E x[6] = {p * p, p * dl, dl * dl, p * q, dl * q, q * q};
-    const E t = warp_sums<6, E>(x, lane);
+    const E t = warp_sums<6>(x, lane);
     if ((lane & 3) == 0 && lane < 24) sm.Gs[wid][lane >> 2] = t;
   }
   __syncthreads();
 }
 
-template <typename E>
-__device__ inline E derived_norm2(const NodesSmem<E>& sm) {
+__device__ inline E derived_norm2(const NodesSmem& sm) {
   // columns of Gs: 0 PP, 1 Pd, 2 dd, 3 PQ, 4 dQ, 5 QQ
   const E* a = sm.Gs[0];
   const E* b = sm.Gs[1];
@@ -494,8 +475,7 @@ __device__ inline E derived_norm2(const NodesSmem<E>& sm) {
 }
 
 // The same in FP32, mag the sum of its terms' magnitudes (clearly_less).
-template <typename E>
-__device__ __forceinline__ float derived_norm2_f32(const NodesSmem<E>& sm, float& mag) {
+__device__ __forceinline__ float derived_norm2_f32(const NodesSmem& sm, float& mag) {
   float a[6], b[6], c[6];
 #pragma unroll
   for (int k = 0; k < 6; k++) a[k] = tof(sm.Gs[0][k]), b[k] = tof(sm.Gs[1][k]), c[k] = tof(sm.Gs[2][k]);
@@ -505,7 +485,7 @@ __device__ __forceinline__ float derived_norm2_f32(const NodesSmem<E>& sm, float
   return p + 2.0f * (x0 + x1 + x2);
 }
 
-template <typename E, int EPT>
+template <int EPT>
 __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
   cg::cluster_group cl = cg::this_cluster();
   const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
@@ -513,7 +493,7 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
   if (q >= a.n_inst) return;  // whole cluster, uniformly
   if (a.active && !a.active[q]) return;
   const InstDev& I = a.inst[q];
-  __shared__ NodesSmem<E> sm;
+  __shared__ NodesSmem sm;
   const int N = a.N, K = N * N * N;
   const double dv = a.dv, wd = a.dv * a.dv * a.dv;
   const E w = cvt<E>(wd);
@@ -606,7 +586,7 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
     E m7[7] = {a0, v1 * a0, v2 * a0, a3, vq12 * a0 + a4, (lw && v1d < 0.0) ? v1 * a0 : zero,
                (rw && v1d > 0.0) ? v1 * a0 : zero};
     double t7[7];
-    cluster_reduce<7, E>(m7, t7, sm, buf, cl, CS);
+    cluster_reduce<7>(m7, t7, sm, buf, cl, CS);
     E mom[5];
 #pragma unroll
     for (int k = 0; k < 5; k++) mom[k] = w * sm.red_tote[k];
@@ -628,7 +608,7 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
       double th0[5];
 #pragma unroll
       for (int k = 0; k < 5; k++) th0[k] = a.theta[5 * (long long)(I.cell0 + j) + k];
-      int n0 = solve_mg<E>(sm, N, w, mom, th0, false, L, ntol, I.newton_max, status);
+      int n0 = solve_mg(sm, N, w, mom, th0, false, L, ntol, I.newton_max, status);
       if (n0 > 0) c_newton += n0;
       c_solves++;
     }
@@ -674,7 +654,7 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
         }
         E v6[6] = {rs, b0, v1 * b0, v2 * b0, b3, vq12 * b0 + b4};
         double t6[6];
-        cluster_reduce<6, E>(v6, t6, sm, buf, cl, CS);
+        cluster_reduce<6>(v6, t6, sm, buf, cl, CS);
         // thread 0 decides: stop, and whether step 1 is attempted (existence test, eq. (26))
         if (tid == 0) {
           const float rf = tof(sm.red_tote[0]);
@@ -693,7 +673,7 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
             if (!(res == res)) sml = 2;
             double sd[5] = {wd * t6[1], wd * t6[2], wd * t6[3], wd * t6[4], wd * t6[5]};
             bool exists = pfp && sd[0] > 0.0 && sd[0] * sd[4] > sd[1] * sd[1] + sd[2] * sd[2] + sd[3] * sd[3];
-            if (pfp && !exists && relax) exists = relax_target<E>(sm, w, sd);
+            if (pfp && !exists && relax) exists = relax_target(sm, w, sd);
             ex = exists;
           }
           sm.ctl = (decide(sml) ? 1 : 0) | (ex ? 2 : 0);
@@ -713,12 +693,12 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
           if (tid < 5) sm.thp[tid] = sm.thg[tid];
           __syncthreads();
           // the last evaluation is M[g]'s: reused as the first one of step 1
-          int n1 = newton_cta<E>(sm, N, w, true, sv, sm.thp, L, ntol, I.newton_max, true);
+          int n1 = newton_cta(sm, N, w, true, sv, sm.thp, L, ntol, I.newton_max, true);
           c_solves++;
           if (n1 >= 0) {
             c_newton += n1;
             used = true;
-            copy_factors<E>(sm, sm.Ep);
+            copy_factors(sm, sm.Ep);
           }
         }
         if (!used) c_fallback++;
@@ -729,7 +709,7 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
       E momP[5];
       if (used) {
         float Aa[15];
-        moments_from_sums<E>(sm.S[0], sm.S[1], sm.S[2], momP, Aa);
+        moments_from_sums(sm.S[0], sm.S[1], sm.S[2], momP, Aa);
 #pragma unroll
         for (int k = 0; k < 5; k++) momP[k] = w * momP[k];
       } else {
@@ -754,22 +734,22 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
       if (!used && tid < 3 * kMaxN) sm.Ep[tid / kMaxN][tid % kMaxN] = sm.Eg[tid / kMaxN][tid % kMaxN];
       E m5[5] = {c0, v1 * c0, v2 * c0, c3, vq12 * c0 + c4};
       double t5[5];
-      cluster_reduce<5, E>(m5, t5, sm, buf, cl, CS);
+      cluster_reduce<5>(m5, t5, sm, buf, cl, CS);
       it++;
       E mm[5];
 #pragma unroll
       for (int k = 0; k < 5; k++) mm[k] = w * sm.red_tote[k];
       // warm start: the step-1 Maxwellian approximates M of the updated iterate
-      int n2 = solve_mg<E>(sm, N, w, mm, used ? sm.thp : sm.thg, eval_at_start, L, ntol, I.newton_max, status);
+      int n2 = solve_mg(sm, N, w, mm, used ? sm.thp : sm.thg, eval_at_start, L, ntol, I.newton_max, status);
       if (n2 > 0) c_newton += n2;
       c_solves++;
       // ---- residual and step-1 target of the new iterate from the step-2 identity
-      derived_sums<E>(sm);
+      derived_sums(sm);
       // warp 0 decides; its lanes form the five components of the step-1 target
       if (tid < 32) {
         const int lane = tid;
-        const E mwk = lane_moment<E>(sm.S1w, sm.S[1], sm.S[2], lane);  // sum phi (|v1|/dx) M[g]
-        const E sk = w * mwk - Acoef * pick5<E>(momP, lane) + Acoef * pick5<E>(mm, lane);
+        const E mwk = lane_moment(sm.S1w, sm.S[1], sm.S[2], lane);  // sum phi (|v1|/dx) M[g]
+        const E sk = w * mwk - Acoef * pick5(momP, lane) + Acoef * pick5(mm, lane);
         if (lane < 5) sm.svE[lane] = sk;
         float mag;
         const float nf = derived_norm2_f32(sm, mag);
@@ -780,7 +760,7 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
         int ex = pfp ? clearly_exists(f[0], f[1], f[2], f[3], f[4]) : 0;
         if (sml < 0 || ex < 0 || (pfp && relax && ex == 0)) {  // in FP64, from the full sums
           const double sdk = tod(sk);
-          double nrm = lane == 5 ? tod(derived_norm2<E>(sm)) : 0.0;
+          double nrm = lane == 5 ? tod(derived_norm2(sm)) : 0.0;
           double sd[5];
 #pragma unroll
           for (int k = 0; k < 5; k++) sd[k] = __shfl_sync(0xffffffffu, sdk, k);
@@ -791,7 +771,7 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
             sml = res < I.inner_tol;
             if (!(res == res)) sml = 2;
             bool exists = pfp && sd[0] > 0.0 && sd[0] * sd[4] > sd[1] * sd[1] + sd[2] * sd[2] + sd[3] * sd[3];
-            if (pfp && !exists && relax) exists = relax_target<E>(sm, w, sd);
+            if (pfp && !exists && relax) exists = relax_target(sm, w, sd);
             ex = exists;
           }
         }
@@ -830,15 +810,15 @@ __global__ void __launch_bounds__(256) k_sweep_nodes(SweepArgs a) {
 // The kernel of a shape (null: not compiled) and its launch configuration.
 const void* nodes_kernel(int ept) {
   switch (ept) {
-    case 2: return (const void*)k_sweep_nodes<dfloat, 2>;
-    case 4: return (const void*)k_sweep_nodes<dfloat, 4>;
-    case 8: return (const void*)k_sweep_nodes<dfloat, 8>;
-    case 12: return (const void*)k_sweep_nodes<dfloat, 12>;
-    case 16: return (const void*)k_sweep_nodes<dfloat, 16>;
-    case 20: return (const void*)k_sweep_nodes<dfloat, 20>;
-    case 24: return (const void*)k_sweep_nodes<dfloat, 24>;
-    case 28: return (const void*)k_sweep_nodes<dfloat, 28>;
-    case 32: return (const void*)k_sweep_nodes<dfloat, 32>;
+    case 2: return (const void*)k_sweep_nodes<2>;
+    case 4: return (const void*)k_sweep_nodes<4>;
+    case 8: return (const void*)k_sweep_nodes<8>;
+    case 12: return (const void*)k_sweep_nodes<12>;
+    case 16: return (const void*)k_sweep_nodes<16>;
+    case 20: return (const void*)k_sweep_nodes<20>;
+    case 24: return (const void*)k_sweep_nodes<24>;
+    case 28: return (const void*)k_sweep_nodes<28>;
+    case 32: return (const void*)k_sweep_nodes<32>;
   }
   return nullptr;
 }
