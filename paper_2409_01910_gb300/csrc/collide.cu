@@ -547,9 +547,9 @@ __global__ void __launch_bounds__(256) k_dft_i1(SpecBufs<T> sb, int N) {
 // by instruction fetch (69 KB of code) at 255 registers and two warps per scheduler, and a
 // version with two shared loads per pair (FP64), whose 127 KB of rows for two warps left half
 // of an SM's schedulers idle. Measured: FP32,
-// 32 cells of 32^3, 1.62 -> 1.55 ms (42 TFLOP/s; 64 registers, 20 warps per SM; now held by
-// operand dispatch, 0.7 stalls per issue); FP64 is at 0.87 of the DFMA rate times 10 flops in 6
-// instructions, its cap. FP32 in packed pairs (fma.rn.f32x2 on outputs i, i + 1) took 1.94 ms: about
+// 32 cells of 32^3, 1.62 -> 1.55 ms (42 TFLOP/s; 64 registers, 20 warps per SM; 0.73 of the issue
+// slots, with 1.9 barrier and 0.8 operand-dispatch stalls per issue); FP64 is at 0.9 of the rate of one
+// instruction per 64 cycles and scheduler, its cap. FP32 in packed pairs (fma.rn.f32x2 on outputs i, i + 1) took 1.94 ms: about
 // one move per packed operand.
 // Four warps do 3/14, 4/14, 4/14, 3/14 of the blocks; every other lane group (or block) takes
 // them in the order 1, 0, 3, 2, so that the SM's schedulers get the same work.
@@ -558,7 +558,8 @@ __global__ void __launch_bounds__(256) k_dft_i1(SpecBufs<T> sb, int N) {
 constexpr int kSumBlocksPerStep = 14;  // blocks of (k3, m3) pairs of a step
 
 // Weights of a step: the valid blocks (kb, c), kb major, c ascending, each [m3][k3] of BK x BK
-// (zero where the pair is not valid).
+// (zero where the pair is not valid: 896 values at N = 32 for 721 pairs, 0.24 more of a table that is
+// 1.9 GB of the 2.5 GB workspace of 64 cells in FP64 and 3.7 of 4.6 GB in the mixed solver).
 __host__ __device__ constexpr int sum_first_block(int kb) { return kb == 0 ? 0 : (kb == 1 ? 3 : (kb == 2 ? 7 : 11)); }
 __host__ __device__ constexpr int sum_weights(int BK) { return kSumBlocksPerStep * BK * BK; }
 

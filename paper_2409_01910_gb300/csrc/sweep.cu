@@ -155,8 +155,10 @@ __device__ __forceinline__ float shfl_i(float v, int lane) { return __shfl_sync(
 __device__ __forceinline__ dfloat shfl_i(dfloat v, int lane) {
   return {__shfl_sync(0xffffffffu, v.hi, lane), __shfl_sync(0xffffffffu, v.lo, lane)};
 }
-// FP64 value of a result that is stored: the float halves become doubles by bit operations
-// (an FP32 subnormal counts as zero), which leaves one FP64 instruction per value.
+// FP64 value of a result that is stored: the float halves become doubles by bit operations, which
+// leaves one FP64 instruction per value. An FP32 subnormal counts as zero (a double-float field
+// ends at 2^-100): widen(), which branches for it, took 2617 -> 2687 us of the scan of 64 cells of
+// 32^3 and 9567 -> 9960 us of an ordering of 64 x 64 cells.
 __device__ __forceinline__ double f2d_bits(float x) {
   const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
   unsigned hi = (u & 0x80000000u) | ((m >> 3) + (m >= 0x7f800000u ? 0x70000000u : 0x38000000u));

@@ -14,8 +14,8 @@
 // cycles (a conversion: 101), is its dearest link. So a decision is taken in FP32 where that leaves
 // no doubt, widening to FP64 is done by integer operations, components are spread over lanes, and a
 // warp sum takes 9 double-float additions (warp_sums) instead of 25 to 35. All of it keeps the bits.
-// A visit of the defect correction (64 cells, 32 velocities): 85 -> 55 us, two iterations of
-// sgs_dc_step 89.4 -> 74.0 ms.
+// A visit of the defect correction (64 cells, 32 velocities): 180 -> 116 us, 203 -> 125 us beside the
+// sums; two iterations of sgs_dc_step 89.4 -> 74.0 ms.
 //
 // One thread-block cluster walks the instance's cells in scan order inside a single launch.
 // Each thread owns EPT consecutive velocity nodes of one pencil (fixed i1, i2) in every cell.
