@@ -779,14 +779,20 @@ __device__ __forceinline__ void df_mul_acc(float xh, float xl, float yh, float y
 // with whole blocks of N = 32 it is 121 KB of code and twice as slow.
 __host__ __device__ constexpr int df_side(int BK) { return BK % 2 == 0 ? BK / 2 : BK; }
 
-// One HB x HB square (KIND as in sum_block); rows of the weights are BK apart.
+// Whether a square's rows m3 are a loop, the window moving by register copies, instead of an unrolled
+// body with a rotating one: squares of 7 (N = 28) are 81 KB of code unrolled, 64 cells of 28^3 took
+// 21.6 ms instead of 12.0; squares of 5 (N = 20) 1.63 ms instead of 1.42. Smaller ones lose by it
+// (4, N = 32: 22.3 -> 25.0 ms; 3, N = 24: 3.94 -> 4.55).
+__host__ __device__ constexpr bool df_loop(int BK) { return df_side(BK) >= 5; }
+
+// One HB x HB square (KIND as in sum_block); rows of the weights are BK apart. LOOP: win[i] meets output
+// i of the current m3, otherwise slot (i - u) mod HB.
 template <int KIND, int BK, int HB>
 __device__ __forceinline__ void sum_block_df(const float* wh, const float* wl, const float4* ra, const float4* rb,
                                              float4 (&win)[HB], float (&rh)[HB], float (&rl)[HB], float (&ih)[HB],
                                              float (&il)[HB]) {
-#pragma unroll
-  for (int u = 0; u < HB; u++) {
-    if (KIND == 0 || (KIND < 0 && u > 0)) win[(HB - u) % HB] = ra[-u * kLanes];
+  constexpr bool kLoop = df_loop(BK);
+  auto row = [&](int u) {
     const float4 bv = rb[u * kLanes];
     float h[HB], l[HB];
     load_weights<float, HB>(wh + u * BK, h);
@@ -794,7 +800,7 @@ __device__ __forceinline__ void sum_block_df(const float* wh, const float* wl, c
 #pragma unroll
     for (int i = 0; i < HB; i++) {
       if ((KIND < 0 && i >= u) || (KIND > 0 && i <= u)) continue;
-      const float4 av = win[(i - u + HB) % HB];
+      const float4 av = win[kLoop ? i : (i - u + HB) % HB];
       // w b = (w b_re, w b_im), leading parts exact
       float brh = h[i] * bv.x, brl = fmaf(h[i], bv.x, -brh);
       brl = fmaf(h[i], bv.y, brl);
@@ -807,6 +813,21 @@ __device__ __forceinline__ void sum_block_df(const float* wh, const float* wl, c
       df_mul_acc(-av.z, -av.w, bih, bil, rh[i], rl[i]);
       df_mul_acc(av.x, av.y, bih, bil, ih[i], il[i]);
       df_mul_acc(av.z, av.w, brh, brl, ih[i], il[i]);
+    }
+  };
+  if constexpr (kLoop) {
+#pragma unroll 1
+    for (int u = KIND < 0 ? 1 : 0; u < HB; u++) {
+#pragma unroll
+      for (int i = HB - 1; i > 0; i--) win[i] = win[i - 1];
+      if (KIND <= 0) win[0] = ra[-u * kLanes];
+      row(u);
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < HB; u++) {
+      if (KIND == 0 || (KIND < 0 && u > 0)) win[(HB - u) % HB] = ra[-u * kLanes];
+      row(u);
     }
   }
 }
@@ -899,7 +920,7 @@ __global__ void __launch_bounds__(128 * (BK / df_side(BK)), 2) k_sum_df(SumDfArg
       sum_block_df<-1, BK, HB>(w, w + PW, ra - cl * HB * kLanes, rb + cl * HB * kLanes, win, rh, rl, ih, il);
     } else {
 #pragma unroll
-      for (int i = 1; i < HB; i++) win[i] = ra[i * kLanes];
+      for (int i = 1; i < HB; i++) win[df_loop(BK) ? i - 1 : i] = ra[i * kLanes];
     }
     const int c1 = min(NB - 1, kb + D - 1);
 #pragma unroll 1
