@@ -563,6 +563,9 @@ constexpr int kSumBlocksPerStep = 14;  // blocks of (k3, m3) pairs of a step
 __host__ __device__ constexpr int sum_first_block(int kb) { return kb == 0 ? 0 : (kb == 1 ? 3 : (kb == 2 ? 7 : 11)); }
 __host__ __device__ constexpr int sum_weights(int BK) { return kSumBlocksPerStep * BK * BK; }
 
+// Whether the FP32 sum of a grid keeps both rows in registers (k_sum_regs).
+__host__ __device__ constexpr bool sum_in_registers(int BK) { return BK <= 5; }
+
 // Weight row of one m3: BK consecutive values by the widest aligned loads.
 template <typename T, int BK>
 __device__ __forceinline__ void load_weights(const T* p, T (&w)[BK]) {
@@ -747,6 +750,130 @@ __global__ void __launch_bounds__(512) k_sum(SumArgs<T> a) {
 #pragma unroll
     for (int i = 0; i < BK; i++)
       if (kb * BK + i < n) out[(kb * BK + i) * kLanes + lane] = make_cplx(accr[i], acci[i]);
+  }
+}
+
+// The FP32 sum of the smaller grids (sum_in_registers): a warp per lane group with both rows of a step in
+// registers and the step fully unrolled. Same units, weights and order of additions as k_sum, so
+// the same bits. A step has few pairs there (91 at N = 12, 271 at N = 20), and the four warps of a
+// group in k_sum lose at its barrier, by the blocks they share unevenly and by the rows that each
+// of them loads; this form loses where its code leaves the instruction cache (721 pairs at N = 32).
+// k_sum -> here: 3000 cells of 8^3 61 -> 40 us, 1000 of 12^3 188 -> 142, 1000 of 16^3 830 -> 751, 64
+// of 20^3 203 -> 181. At N = 24 k_sum is the better one for most cell counts (96: 0.87 against 1.08 ms, 200:
+// 1.97 against 2.20, 64: 0.55 against 0.53).
+template <int BK>
+__global__ void __launch_bounds__(128) k_sum_regs(SumArgs<float> a) {
+  constexpr int H = 2 * BK - 1, n = 4 * BK - 1;
+  constexpr int PW = (sum_weights(BK) + 3) / 4 * 4;
+  constexpr int kRow = n * kLanes;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  float* Wb = (float*)smraw;                              // [2][PW]
+  float2* rows = (float2*)(smraw + 2 * PW * sizeof(float));  // [NW][2][n][32]
+  __shared__ __align__(8) uint64_t bar[2];
+  __shared__ int s_err;
+
+  const int NW = blockDim.x >> 5;
+  const int4 ud = a.units[blockIdx.x];  // k1, k2, m1_lo, m1_hi
+  const long long step0 = a.unit_step0[blockIdx.x];
+  const int k1 = ud.x, k2 = ud.y, m1lo = ud.z, m1hi = ud.w;
+  const int m2lo = max(-H, k2 - H), m2hi = min(H, k2 + H);
+  const int nm2 = m2hi - m2lo + 1;
+  const int S = (m1hi - m1lo + 1) * nm2;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g0 = blockIdx.y * NW;
+  const int ng = min(NW, a.G - g0);
+  const uint32_t row_bytes = kRow * sizeof(float2);
+
+  if (a.active) {
+    // a block whose lane groups hold no cell of an active instance has nothing to compute
+    const int c = (g0 + warp) * kLanes + lane;
+    if (!__syncthreads_or(warp < ng && c < a.C && a.active[a.cell_inst[c]])) return;
+  }
+  if (threadIdx.x == 0) {
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
+    s_err = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();
+
+  auto issue = [&](int s) {
+    const int m1 = m1lo + s / nm2, m2 = m2lo + s % nm2, b = s & 1;
+    mbar_arrive_expect_tx(&bar[b], PW * sizeof(float) + ng * 2 * row_bytes);
+    bulk_g2s(Wb + b * PW, a.W + (step0 + s) * PW, PW * sizeof(float), &bar[b]);
+    for (int w = 0; w < ng; w++) {
+      const long long ga = (((long long)(g0 + w) * n + (k1 - m1 + H)) * n + (k2 - m2 + H)) * kRow;
+      const long long gb = (((long long)(g0 + w) * n + (m1 + H)) * n + (m2 + H)) * kRow;
+      float2* dst = rows + w * 2 * kRow;
+      bulk_g2s(dst, a.ahat + ga, row_bytes, &bar[b]);
+      bulk_g2s(dst + kRow, a.bhat + gb, row_bytes, &bar[b]);
+    }
+  };
+
+  if (threadIdx.x == 0 && S > 0) issue(0);
+
+  float accr[n], acci[n];
+#pragma unroll
+  for (int i = 0; i < n; i++) accr[i] = acci[i] = 0.0f;
+
+  const bool active = warp < ng;
+  int fail_b = 0, fail_par = 0;
+  for (int s = 0; s < S; s++) {
+    const int b = s & 1;
+    if (!mbar_wait(&bar[b], (s >> 1) & 1, a.spin_max)) {
+      s_err = 1;
+      fail_b = b;
+      fail_par = (s >> 1) & 1;
+    }
+    float2 Ar[n], Br[n];
+    if (active) {
+      const float2* rw = rows + warp * 2 * kRow + lane;
+#pragma unroll
+      for (int i = 0; i < n; i++) {
+        Ar[i] = rw[i * kLanes];
+        Br[i] = rw[kRow + i * kLanes];
+      }
+    }
+    __syncthreads();
+    if (s_err) break;
+    // every row is in registers: the next step's come into the same buffer
+    if (threadIdx.x == 0 && s + 1 < S) issue(s + 1);
+    if (active) {
+      const float4* W4 = (const float4*)(Wb + b * PW);
+      float4 wv;
+      int have = -1;  // the quad of weights in wv
+#pragma unroll
+      for (int kb = 0; kb < 4; kb++)
+#pragma unroll
+        for (int c = (kb > 2 ? kb - 2 : 0); c <= (kb < 1 ? 2 : 3); c++)
+#pragma unroll
+          for (int t = 0; t < BK * BK; t++) {
+            const int p = (sum_first_block(kb) + c - (kb > 2 ? kb - 2 : 0)) * BK * BK + t;
+            const int m = c * BK + t / BK, k = kb * BK + t % BK, l = k - m + H;
+            if (k >= n || m >= n || l < 0 || l >= n) continue;
+            if (p / 4 != have) wv = W4[p / 4];
+            have = p / 4;
+            const float w = p % 4 == 0 ? wv.x : (p % 4 == 1 ? wv.y : (p % 4 == 2 ? wv.z : wv.w));
+            const float br = w * Br[m].x, bi = w * Br[m].y;
+            accr[k] = fmaf(Ar[l].x, br, accr[k]);
+            accr[k] = fmaf(-Ar[l].y, bi, accr[k]);
+            acci[k] = fmaf(Ar[l].x, bi, acci[k]);
+            acci[k] = fmaf(Ar[l].y, br, acci[k]);
+          }
+    }
+  }
+  if (s_err) {
+    // the failing thread waits (again bounded) for its copies in flight
+    if (threadIdx.x == 0) {
+      atomicOr(&a.cnt[0].status, SGS_ST_TIMEOUT);
+      mbar_wait(&bar[fail_b], fail_par, a.spin_max);
+    }
+    return;
+  }
+  if (active) {
+    float2* out = a.partial + ((long long)blockIdx.x * a.Gs + (g0 + warp)) * kRow;
+#pragma unroll
+    for (int i = 0; i < n; i++) out[i * kLanes + lane] = make_float2(accr[i], acci[i]);
   }
 }
 
@@ -1369,7 +1496,17 @@ static cudaError_t launch_sum_t(const SumArgs<T>& a, int NW, int n_units, cudaSt
       return a.fold == 4 ? launch_sum_f<T, BK, 4>(x, 1, n_units, st) : launch_sum_f<T, BK, 2>(x, 1, n_units, st);
     }
   }
-  return launch_sum_f<T, BK, 1>(a, NW, n_units, st);
+  if constexpr (sizeof(T) == 4 && sum_in_registers(BK)) {
+    constexpr size_t row_bytes = (size_t)2 * (4 * BK - 1) * kLanes * sizeof(float2);
+    const int nw = std::min(NW, a.G);
+    const size_t smem = 2 * sum_pad(2 * BK - 1, 4) * sizeof(float) + nw * row_bytes;
+    cudaError_t e = func_attr((const void*)k_sum_regs<BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_sum_regs<BK><<<dim3(n_units, (a.G + nw - 1) / nw), nw * 32, smem, st>>>(a);
+    return cudaGetLastError();
+  } else {
+    return launch_sum_f<T, BK, 1>(a, NW, n_units, st);
+  }
 }
 
 int sum_pad(int H, int elem_bytes) {
