@@ -337,7 +337,8 @@ typedef struct {
  * there for the reported cluster and threads. The timed scans are real SGS scans: f advances by
  * (reps + 1) symmetric sweeps with the given P per candidate. Then times the spectral sum
  * (the handle's arithmetic, all cells, two launches after one untimed one) for every
- * decomposition of 1, 2 or 4 lane groups per block and about 1500, 3000 or 6000 blocks, and
+ * decomposition of 1, 2 or 4 lane groups per block (FP64 always launches one; there they
+ * divide the work units only) and about 1500, 3000 or 6000 blocks, and
  * keeps the fastest for all later collision steps (the sums write only workspace buffers;
  * the reduction order of the partial sums follows the decomposition, so results may differ
  * in the last bits). Synchronises the stream; not graph-capturable (call it before

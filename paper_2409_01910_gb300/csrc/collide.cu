@@ -1457,7 +1457,10 @@ static size_t dft_smem(int N, int extra_cplx, int extra_real) {
 }
 
 // Lane groups per block of a sum over `groups` of them that takes F steps at once: as many as asked
-// for, within an SM's shared memory.
+// for, within an SM's shared memory; one in FP64, where eight warps that wait for each other at a
+// step's barrier leave the pipe idle more than four (two groups a block against one: 200 cells of 8^3 98
+// against 87 us, 64 of 12^3 347 and 322, of 24^3 21.4 and 21.3 ms, of 32^3 128.4 and 126.8; the other way at
+// 64 cells of 20^3, 6.81 and 6.88). The units don't follow it, so the bits don't either.
 static size_t sum_group_bytes(int BK, int elem_bytes) {
   return (size_t)2 * (2 * (4 * BK - 1) + 1) * kLanes * 2 * elem_bytes;
 }
@@ -1466,7 +1469,7 @@ static size_t sum_weight_bytes(int BK, int elem_bytes, int F) {
 }
 static int sum_groups(int BK, int elem_bytes, int F, int NW, int groups) {
   const int fit = (int)((220 * 1024 - sum_weight_bytes(BK, elem_bytes, F)) / sum_group_bytes(BK, elem_bytes));
-  return std::max(1, std::min(std::min(NW, groups), fit));
+  return std::max(1, std::min(std::min(elem_bytes == 8 ? 1 : NW, groups), fit));
 }
 
 template <typename T, int BK, int F>
