@@ -542,7 +542,8 @@ __global__ void __launch_bounds__(256) k_dft_i1(SpecBufs<T> sb, int N) {
 // registers and walks the blocks c of m3: |kb - c| <= 1 is a full BK x BK square of valid pairs
 // (|k3 - m3| <= H), |kb - c| = 2 a triangle, |kb - c| = 3 empty. Along m3 the BK values of ahat
 // that meet the outputs slide by one, so a thread loads one value of each row per m3 and keeps
-// the window in registers (its slots rotate; the loop is unrolled by BK). This replaces a
+// the window in registers (its slots rotate; the loop is unrolled by BK). In FP32 this is the form for
+// N >= 24 (k_sum_regs below that). It replaces a
 // fully unrolled step of 721 pairs per warp with both rows in registers (FP32), which was bound
 // by instruction fetch (69 KB of code) at 255 registers and two warps per scheduler, and a
 // version with two shared loads per pair (FP64), whose 127 KB of rows for two warps left half
